@@ -390,9 +390,9 @@ dh_status dh_graph_stage_times(dh_plan* plan, float* ms_out, int32_t n);
  *                  the persistent grid and the 32x8 columns with the register
  *                  cap only (20 to 48 candidates);
  *   FV2 (scheme 2): the three variants of dh_plan_set_variant_muscl;
- *   FD (scheme 1): register cap x shared-memory staging by plain loads or by
- *                  TMA tensor copies (2 candidates, or 6 with TMA -- 4 for
- *                  GW59; TMA only when every level is a run of back-to-back
+ *   FD (scheme 1): register cap x staging by asynchronous copies a variable at
+ *                  a time or by TMA tensor copies (2 candidates, or 6 with TMA --
+ *                  4 for GW59; TMA only when every level is a run of back-to-back
  *                  patches, see dh_plan_set_variant).
  * `out` is overwritten.  If cache_path is NULL the environment variable
  * DH_TUNE_CACHE names the cache file (no cache when it is unset).  With a cache
@@ -428,11 +428,13 @@ dh_status dh_autotune_steps(dh_plan* plan, int32_t scheme, int32_t rk, int32_t n
  * shape 1 and bit 5 need bit 1, bit 5 excludes bit 2 and tile shapes 2 and 3,
  * tile shape 3 excludes bit 2; DH_EINVAL otherwise), fv_zs 0..1 (z-chunks of <= 16 planes,
  * and a thin last wave filled with half-height chunks of the cheapest columns), fd_var
- * 0, 2, 4 or 6 (bit 1: two CTAs per SM; bit 2: TMA staging, which needs every
- * run of equal-size patches to be stored back to back with its face
- * neighbours inside the run; DH_EUNSUPPORTED otherwise), or, for systems of
- * at most five variables (not GW59), 12 / 20: TMA staging with register caps
- * for three / four CTAs per SM. */
+ * 0, 2, 4 or 6 (bit 1: two CTAs per SM, else three; bit 2: TMA staging, which
+ * needs every run of equal-size patches to be stored back to back with its
+ * face neighbours inside the run; DH_EUNSUPPORTED otherwise), or, for systems
+ * of at most five variables (not GW59), 12 / 20: TMA staging with register
+ * caps for three / four CTAs per SM.  TMA staging is compiled for the wave
+ * system: the others run the asynchronous copies for these values, and GW59
+ * has one form for all of them. */
 dh_status dh_plan_set_variant(dh_plan* plan, int32_t fv_var, int32_t fv_zs, int32_t fd_var);
 
 /* Variant of the second-order FV stage (patch_update_fv_muscl), also chosen by

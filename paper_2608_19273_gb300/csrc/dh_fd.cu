@@ -5,31 +5,35 @@
 //   dQ/dx  = [(Q_-2 - Q_+2) + 8 (Q_+1 - Q_-1)] / (12 dx)
 //   delta6 = Q_-3 - 6 Q_-2 + 15 Q_-1 - 20 Q_0 + 15 Q_+1 - 6 Q_+2 + Q_+3
 //   out = a q0 + b qs + g dt L ; acc += d dt L
-// The three directional sixth differences are summed grouped by distance r
-// (T_r = sum_d (Q_-r + Q_+r) - 6 Q_0, with 6 Q_0 formed by the same additions),
-// which is exactly zero on constant data, so constant states stay bitwise
-// constant.
+// Constant states stay bitwise constant (the weights of every stencil sum to zero, and equal
+// terms cancel exactly).
 //
-// Kernel design: a CTA owns an 8x8x4 tile of one patch (one voxel per
-// thread).  The variables are staged in groups of at most five into shared
-// memory together with the tile's three-voxel face halos (edges and corners
-// are never read by the axis-aligned stencils and are not loaded); halo
-// voxels outside the patch come from the face neighbours.  Two staging
-// variants exist (the autotuner picks one):
-//   * plain loads: every thread copies voxels into a padded 14x14x10 box;
-//   * TMA: one thread issues seven 5-D tensor copies per group (interior box
-//     and six face slabs, from this patch or its neighbours) that complete on
-//     an mbarrier; groups are double buffered, so the next field group of
-//     GW59 streams in while the current one is computed.
-// Every derivative is taken only for the variables that a column of B_d
-// reads.  GW59 is processed field by field (lapse/shift first, then the 11
-// scalar-wave fields), keeping per voxel only the coupling quantities (alpha,
-// beta, grad alpha, phi_b Pi_b, source sums) in registers.
+// Kernel design: a CTA owns an 8x8x4 tile of one patch, one voxel per thread.  The FP64 pipe
+// (2 lanes per clock and SM) was the bound of this stage when the stencils were FP64 sums: 23 operations
+// for the sixth differences of a variable and 3 per derivative, of 160 (wave) and 2400 (GW59) a
+// voxel.  They are now sums in 64-bit fixed point on the integer pipe (dh_fixed.cuh, fd_stencil),
+// which the FP64 operations of the products and of the update run beside: 39 and 948 FP64
+// instructions a voxel are left, a fifth of them conversions at a third of an FMA's cost.
+// Each variable with the tile's three-voxel face halos (edges and corners are never read by the
+// axis-aligned stencils) is brought into a padded 14x14x10 box of shared memory by asynchronous
+// copies, several variables ahead of its use (FdRing), so one barrier per variable is all the
+// waiting there is; halo voxels outside the patch come from the face neighbours.  A variable's
+// update is written after the next variable's staging: its chain of FP64 operations (64 clocks each)
+// is then issued among the integer operations of the next stencil.
+// Measured per RK4 step: the wave system on 8.4 M voxels 17.9 -> 4.4 ms (39% of the time the FP64
+// operations alone take, half of the issue slots; 0.9 ms would be the memory's), GW59 on
+// 3.9 M voxels 97 -> 30.5 ms (FP64 pipe: 70% busy).  With the sums in FP64 and every variable staged by plain
+// loads: 12 and 75 ms at best.  Fixed point with the boxes loaded a group of five at a time: 5.7 and 36.9;
+// TMA copies of dense boxes (no padding, so every neighbour's address takes selects): 5.2 for the wave
+// system, kept as a variant for it.
+// GW59 goes variable by variable (lapse and shift first, then the 11 scalar-wave fields), keeping
+// per voxel only the coupling quantities (alpha, beta, grad alpha, phi_b Pi_b, source sums) in registers.
 #include <cuda.h>
 
 #include <cstring>
 #include <type_traits>
 
+#include "dh_fixed.cuh"
 #include "dh_internal.cuh"
 #include "dh_pde.cuh"
 
@@ -52,9 +56,12 @@ struct FdArgs {
   const double* q0;
   double* out;
   double* acc;
+  const double* acc_in;            // acc = acc_in + d dt L (acc itself, or the state the sum starts from)
+  double* acc_copy;                // NULL, or a second array that receives the new acc
   const double* mat;
   const double* dt_dev;
   double a, b, g, d;
+  int a1, b1, b0;                  // a == 1, b == 1, b == 0 (host side: a comparison is an FP64 operation)
   double sigma;
   double* lam_out;
   unsigned long long* red;
@@ -131,19 +138,15 @@ __device__ __forceinline__ void fd_slot(int s, int& x, int& y, int& z) {
 __device__ __forceinline__ int fd_box(int x, int y, int z) { return ((z + FH) * FBY + (y + FH)) * FBX + (x + FH); }
 
 // ------------------------------------------------------------- stencils
-// 4th-order centred derivative (times 1/(12 dx)) from the values at -2, -1, +1, +2.
-__device__ __forceinline__ double st_d1(const DevParams& P, double m2, double m1, double p1, double p2, double r12) {
-  return PMUL(P, fma(8.0, PSUB(P, p1, m1), PSUB(P, m2, p2)), r12);
-}
-// Read access to one staged group: the padded box ...
+// Read access to one staged variable in a padded box (the variable index is not used: the box
+// holds one) ...
 struct BoxAcc {
-  const double* box;
-  int c;
-  __device__ double val(int v) const { return box[v * FBOX + c]; }
+  const double* c;  // this voxel's slot
+  __device__ double val(int) const { return *c; }
   template <int D>
-  __device__ double nb(int v, int o) const {
+  __device__ double nb(int, int o) const {
     constexpr int st = D == 0 ? 1 : (D == 1 ? FBX : FBX * FBY);
-    return box[v * FBOX + c + o * st];
+    return c[o * st];
   }
 };
 
@@ -173,44 +176,82 @@ struct TmaAcc {
   }
 };
 
-template <int D, class Acc>
-__device__ __forceinline__ double acc_d1(const DevParams& P, const Acc& S, int v, double r12) {
-  return st_d1(P, S.template nb<D>(v, -2), S.template nb<D>(v, -1), S.template nb<D>(v, 1), S.template nb<D>(v, 2), r12);
-}
-// Sum over the three directions of the sixth differences, grouped by distance:
+// The linear stencils of one variable at one voxel: the sum of the sixth differences and the
+// unscaled derivatives (q_-2 - q_+2) + 8 (q_+1 - q_-1) along x, y, z.
+struct Stencil {
+  double ko, d[3];
+};
+
+// In FP64 operations, for values that the fixed-point form does not take (infinite, NaN, or beyond
+// its exponents); x[d]: the values at -3, -2, -1, +1, +2, +3 along d.  The sixth differences are
+// grouped by distance,
 //   sum_d delta6_d = T3 - 6 T2 + 15 T1,   T_r = S_r - 6c,
 //   S_r = ((Q_-r + Q_+r)_x + (Q_-r + Q_+r)_y) + (Q_-r + Q_+r)_z,
-// with 6c formed as ((2c + 2c) + 2c) -- the very additions S_r performs on
-// constant data -- so every T_r is exactly 0 on constants (23 FP64 operations
-// per variable instead of 27 for three bracketed directional differences).
-template <class Acc>
-__device__ __forceinline__ double acc_ko3(const DevParams& P, const Acc& S, int v) {
-  const double c = S.val(v);
-  const double two = PMUL(P, 2.0, c);
-  const double six = PADD(P, PADD(P, two, two), two);
+// with 6c formed as ((2c + 2c) + 2c) -- the very additions S_r performs on constant data -- so
+// every T_r is exactly 0 on constants (23 FP64 operations).  A stencil of zeros, common in fields
+// that start from rest, gives zeros at once.
+template <int DM>
+__device__ __forceinline__ Stencil fd_stencil_fp64(double c, const double (&x)[3][6]) {
+  long long any = __double_as_longlong(c);
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) any |= __double_as_longlong(x[d][i]);
+  Stencil R{0.0, {0.0, 0.0, 0.0}};
+  if ((any & 0x7fffffffffffffffll) == 0) return R;
+  const double two = 2.0 * c, six = (two + two) + two;
   double T[3];
 #pragma unroll
-  for (int r = 1; r <= 3; ++r) {
-    const double sx = PADD(P, S.template nb<0>(v, -r), S.template nb<0>(v, r));
-    const double sy = PADD(P, S.template nb<1>(v, -r), S.template nb<1>(v, r));
-    const double sz = PADD(P, S.template nb<2>(v, -r), S.template nb<2>(v, r));
-    T[r - 1] = PSUB(P, PADD(P, PADD(P, sx, sy), sz), six);
+  for (int r = 1; r <= 3; ++r)
+    T[r - 1] = (((x[0][3 - r] + x[0][2 + r]) + (x[1][3 - r] + x[1][2 + r])) + (x[2][3 - r] + x[2][2 + r])) - six;
+  R.ko = fma(15.0, T[0], fma(-6.0, T[1], T[2]));
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    if (DM & (1 << d)) R.d[d] = fma(8.0, x[d][3] - x[d][2], x[d][1] - x[d][4]);
+  return R;
+}
+
+// In fixed point (dh_fixed.cuh): the 19 values are aligned once and serve all four sums, whose
+// weights are small integers (192 by magnitude for the sixth differences: eight bits above the
+// significand, which leaves two guard bits).  About 300 integer instructions and one conversion
+// per sum instead of 23 FP64 operations and 3 per derivative: bound by the integer pipe, which the
+// FP64 operations of the terms run beside.  The error of the sixth differences is below that
+// of the FP64 sums, which round at partial sums of up to eight times the values and then weigh them
+// by 15.  DM: bit d for the derivative along d.
+template <int DM, class Acc>
+__device__ __forceinline__ Stencil fd_stencil(const Acc& S, int v) {
+  constexpr int SH = 2;
+  double x[3][6];  // values at -3, -2, -1, +1, +2, +3
+  const double c = S.val(v);
+  int e = fx_exp(c);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int o = i < 3 ? i - 3 : i - 2;
+    x[0][i] = S.template nb<0>(v, o);
+    x[1][i] = S.template nb<1>(v, o);
+    x[2][i] = S.template nb<2>(v, o);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) e = max(e, fx_exp(x[d][i]));
   }
-  return fma(15.0, T[0], fma(-6.0, T[1], T[2]));
+  if (!fx_ok(e)) return fd_stencil_fp64<DM>(c, x);
+  long long s[3] = {0, 0, 0};  // S_1, S_2, S_3
+  Stencil R{0.0, {0.0, 0.0, 0.0}};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    long long m[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) m[i] = fx_align<SH>(x[d][i], e);
+    s[0] += m[2] + m[3];
+    s[1] += m[1] + m[4];
+    s[2] += m[0] + m[5];
+    if (DM & (1 << d)) R.d[d] = fx_value<SH>(((m[3] - m[2]) << 3) + (m[1] - m[4]), e);
+  }
+  const long long t = (s[2] - 6 * s[1]) + (15 * s[0] - 60 * fx_align<SH>(c, e));
+  R.ko = fx_value<SH>(t, e);
+  return R;
 }
 
 // ------------------------------------------------------------- staging
-// Plain loads into the padded box (single buffer; the caller synchronises).
-__device__ __forceinline__ void fd_stage_vars(const FdArgs& A, double* box, const FdWork& w, int p, int v0, int nv) {
-  for (int s = threadIdx.x; s < FNSLOT; s += FNT) {
-    int x, y, z;
-    fd_slot(s, x, y, z);
-    const int64_t e = fd_vox_index(A.patches, w.patch, p, w.x0 + x, w.y0 + y, w.z0 + z);
-    const int c = fd_box(x, y, z);
-    for (int v = 0; v < nv; ++v) box[v * FBOX + c] = __ldg(A.qs + (int64_t)(v0 + v) * A.vs + e);
-  }
-}
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -279,64 +320,123 @@ __device__ bool tma_wait_all(const FdArgs& A, uint64_t* bar, uint32_t parity) {
   return true;
 }
 
+// Ring of NB padded boxes, one variable each: while variable i is computed, the copies of the
+// next NB - 1 variables are in flight (asynchronous 8-byte copies global -> shared, one commit
+// group per variable; every thread copies the same four of the 1024 slots of every variable, so
+// their indexes are formed once per tile).  One barrier per variable.
+static_assert(FNSLOT == 4 * FNT, "four slots per thread");
+template <int NB>
+struct FdRing {
+  double* box;         // NB x FBOX doubles of shared memory
+  const double* qs;
+  int64_t vs, e[4];    // arena elements of this thread's slots within a variable
+  int c[4];            // their slots in a box
+  int centre;
+
+  __device__ __forceinline__ FdRing(const FdArgs& A, const FdWork& w, int p, double* smem) : box(smem), qs(A.qs), vs(A.vs) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      int x, y, z;
+      fd_slot(threadIdx.x + k * FNT, x, y, z);
+      e[k] = fd_vox_index(A.patches, w.patch, p, w.x0 + x, w.y0 + y, w.z0 + z);
+      c[k] = fd_box(x, y, z);
+    }
+    centre = c[0];  // slot 0 of a thread is its own voxel
+  }
+  // The copies of variable v into box b (v < 0: an empty group, so that the count of groups in
+  // flight stays the same to the end).
+  __device__ __forceinline__ void issue(int v, int b) {
+    if (v >= 0) {
+      const double* src = qs + (int64_t)v * vs;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(box + b * FBOX + c[k])),
+                     "l"(src + e[k])
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  // Waits for the oldest group but NB - 2: after the barrier variable i of the sequence is in its
+  // box and every thread has left the box of variable i - 1, which the next copies overwrite.
+  __device__ __forceinline__ void wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(NB - 2) : "memory");
+    __syncthreads();
+  }
+  __device__ __forceinline__ BoxAcc acc(int b) const { return BoxAcc{box + b * FBOX + centre}; }
+};
+
+// What the update of one variable reads from memory, loaded ahead of its use.
+struct FdOld {
+  double q0, acc;
+};
+__device__ __forceinline__ FdOld fd_old(const FdArgs& A, int64_t ev) {
+  FdOld o{0.0, 0.0};
+  if (A.out && A.q0) o.q0 = __ldg(A.q0 + ev);
+  if (A.acc && A.acc_in != A.qs) o.acc = A.acc_in[ev];
+  return o;
+}
+
 // out / acc update of one variable; returns the new value of the result.
-__device__ __forceinline__ double fd_combine(const FdArgs& A, int64_t ev, double qsv, double L, double gdt,
+__device__ __forceinline__ double fd_combine(const FdArgs& A, int64_t ev, const FdOld& o, double qsv, double L, double gdt,
                                              double ddt) {
   double res = 0.0;
   if (A.out) {
-    double base = A.b == 1.0 ? qsv : PMUL(A.P, A.b, qsv);
-    if (A.q0) base = fma(A.a, __ldg(A.q0 + ev), base);
+    double base;
+    if (A.q0 && A.b0 && A.a1) {
+      base = o.q0;
+    } else {
+      base = A.b1 ? qsv : PMUL(A.P, A.b, qsv);
+      if (A.q0) base = fma(A.a, o.q0, base);
+    }
     res = fma(gdt, L, base);
   }
   if (A.acc) {
-    const double r = fma(ddt, L, A.acc[ev]);
+    const double r = fma(ddt, L, A.acc_in == A.qs ? qsv : o.acc);
     A.acc[ev] = r;
+    if (A.acc_copy) A.acc_copy[ev] = r;
     if (!A.out) res = r;
   }
   if (A.out) A.out[ev] = res;
   return res;
 }
 
+// The tile's scalars, formed once per CTA (a division takes about nine FP64 operations).
+struct FdScalars {
+  double r12, ko, gdt, ddt;  // 1/(12 dx), sigma/(64 dx), g dt, d dt
+};
+__device__ __forceinline__ void fd_scalars(const FdArgs& A, double dx, FdScalars* s) {
+  if (threadIdx.x == 0) {
+    const double dt = *A.dt_dev;
+    s->r12 = 1.0 / (12.0 * dx);
+    s->ko = A.sigma / (64.0 * dx);
+    s->gdt = A.g * dt;
+    s->ddt = A.d * dt;
+  }
+}
+
 // ------------------------------------------------------------- generic (N <= 5)
-template <class PDE, class Acc>
-__device__ void fd_voxel_generic(const FdArgs& A, const Acc& S, int64_t e, double dx, double& lam_thread) {
+// Stencils of all variables of a system by its B (dq: derivatives times 1/(12 dx) where a column
+// of B_d reads them), then the update.
+template <class PDE>
+__device__ __forceinline__ void fd_finish_generic(const FdArgs& A, const double* q, const double* ko, double (&dq)[3][PDE::N],
+                                                  int64_t e, const FdScalars& C, double& lam_thread) {
   constexpr int N = PDE::N, NV = PDE::N + PDE::M;
-  const double r12 = 1.0 / (12.0 * dx);
-  const double ko = A.sigma / (64.0 * dx);
-  const double dt = *A.dt_dev;
-  const double gdt = A.g * dt, ddt = A.d * dt;
-  double q[NV], L[N], W[1];
-#pragma unroll
-  for (int v = 0; v < N; ++v) q[v] = S.val(v);
-#pragma unroll
-  for (int v = 0; v < PDE::M; ++v) q[N + v] = __ldg(A.mat + (int64_t)v * A.vs + e);
+  double L[N], W[1], D[N], res[NV];
   if (PDE::SRC) PDE::source(q, W, A.P, L);
   else {
 #pragma unroll
     for (int v = 0; v < N; ++v) L[v] = 0.0;
   }
-  double dq[N], D[N];
 #pragma unroll
-  for (int v = 0; v < N; ++v) dq[v] = PDE::needs_grad(0, v) ? acc_d1<0>(A.P, S, v, r12) : 0.0;
-  PDE::ncp(0, q, dq, A.P, D);
+  for (int d = 0; d < 3; ++d) {
+    PDE::ncp(d, q, dq[d], A.P, D);
 #pragma unroll
-  for (int v = 0; v < N; ++v) L[v] = PSUB(A.P, L[v], D[v]);
-#pragma unroll
-  for (int v = 0; v < N; ++v) dq[v] = PDE::needs_grad(1, v) ? acc_d1<1>(A.P, S, v, r12) : 0.0;
-  PDE::ncp(1, q, dq, A.P, D);
-#pragma unroll
-  for (int v = 0; v < N; ++v) L[v] = PSUB(A.P, L[v], D[v]);
-#pragma unroll
-  for (int v = 0; v < N; ++v) dq[v] = PDE::needs_grad(2, v) ? acc_d1<2>(A.P, S, v, r12) : 0.0;
-  PDE::ncp(2, q, dq, A.P, D);
-#pragma unroll
-  for (int v = 0; v < N; ++v) L[v] = PSUB(A.P, L[v], D[v]);
-  double res[NV];
-#pragma unroll
-  for (int v = 0; v < N; ++v) {
-    const double Lv = fma(ko, acc_ko3(A.P, S, v), L[v]);
-    res[v] = fd_combine(A, (int64_t)v * A.vs + e, q[v], Lv, gdt, ddt);
+    for (int v = 0; v < N; ++v) L[v] = PSUB(A.P, L[v], D[v]);
   }
+#pragma unroll
+  for (int v = 0; v < N; ++v)
+    res[v] = fd_combine(A, (int64_t)v * A.vs + e, fd_old(A, (int64_t)v * A.vs + e), q[v], fma(C.ko, ko[v], L[v]),
+                        C.gdt, C.ddt);
   if (A.lam_out) {
 #pragma unroll
     for (int v = N; v < NV; ++v) res[v] = q[v];
@@ -345,56 +445,106 @@ __device__ void fd_voxel_generic(const FdArgs& A, const Acc& S, int64_t e, doubl
   }
 }
 
-// The wave system written out (same operator as the generic path with
-// PdeWave's B and S): the 1/(12 dx) of the derivatives is folded into the
-// FMAs that consume them.
+// The wave system written out (same operator as the generic path with PdeWave's B and S): the
+// 1/(12 dx) of the derivatives is folded into the FMAs that consume them.
 //   L_phi   = Pi + KO,   L_Pi = c^2 r12 (Dx psi_x + Dy psi_y + Dz psi_z) - damp Pi + KO,
 //   L_psi_d = r12 Dd Pi + KO,   Dd q = (q_-2 - q_+2) + 8 (q_+1 - q_-1) along d.
-template <int D, class Acc>
-__device__ __forceinline__ double acc_raw(const DevParams& P, const Acc& S, int v) {
-  return fma(8.0, PSUB(P, S.template nb<D>(v, 1), S.template nb<D>(v, -1)),
-             PSUB(P, S.template nb<D>(v, -2), S.template nb<D>(v, 2)));
-}
-
-template <class Acc>
-__device__ void fd_voxel_wave(const FdArgs& A, const Acc& S, int64_t e, double dx, double& lam_thread) {
+// `stage(v)` gives access to variable v once it is staged; it is called once per variable, in the
+// order 1, 2, 3, 4, 0.
+// A variable's update stands after the staging of the next one, so that its FP64 operations can be
+// issued among the integer operations of the next stencil.
+template <class Stage>
+__device__ __forceinline__ void fd_voxel_wave(const FdArgs& A, Stage stage, int64_t e, const FdScalars& C, double& lam_thread) {
   const DevParams& P = A.P;
-  const double r12 = 1.0 / (12.0 * dx);
-  const double ko = A.sigma / (64.0 * dx);
-  const double dt = *A.dt_dev;
-  const double gdt = A.g * dt, ddt = A.d * dt;
-  const double q[5] = {S.val(0), S.val(1), S.val(2), S.val(3), S.val(4)};
   const double c = __ldg(A.mat + e);
-  const double div = PADD(P, PADD(P, acc_raw<0>(P, S, 2), acc_raw<1>(P, S, 3)), acc_raw<2>(P, S, 4));
-  double L[5];
-  L[0] = fma(ko, acc_ko3(P, S, 0), q[1]);
-  L[1] = fma(ko, acc_ko3(P, S, 1), fma(PMUL(P, PMUL(P, c, c), r12), div, PMUL(P, -P.damp, q[1])));
-  L[2] = fma(ko, acc_ko3(P, S, 2), PMUL(P, r12, acc_raw<0>(P, S, 1)));
-  L[3] = fma(ko, acc_ko3(P, S, 3), PMUL(P, r12, acc_raw<1>(P, S, 1)));
-  L[4] = fma(ko, acc_ko3(P, S, 4), PMUL(P, r12, acc_raw<2>(P, S, 1)));
-#pragma unroll
-  for (int v = 0; v < 5; ++v) fd_combine(A, (int64_t)v * A.vs + e, q[v], L[v], gdt, ddt);
+  const int64_t vs = A.vs;
+  Stencil sp, s1, s2, s3;
+  double Pi, q1, q2, q3, div;
+  const FdOld o1 = fd_old(A, vs + e);
+  {
+    const auto S = stage(1);
+    Pi = S.val(1);
+    sp = fd_stencil<7>(S, 1);
+  }
+  const FdOld o2 = fd_old(A, 2 * vs + e);
+  {
+    const auto S = stage(2);
+    q1 = S.val(2);
+    s1 = fd_stencil<1>(S, 2);
+  }
+  const FdOld o3 = fd_old(A, 3 * vs + e);
+  {
+    const auto S = stage(3);
+    fd_combine(A, 2 * vs + e, o2, q1, fma(C.ko, s1.ko, PMUL(P, C.r12, sp.d[0])), C.gdt, C.ddt);
+    q2 = S.val(3);
+    s2 = fd_stencil<2>(S, 3);
+    div = PADD(P, s1.d[0], s2.d[1]);
+  }
+  const FdOld o4 = fd_old(A, 4 * vs + e);
+  {
+    const auto S = stage(4);
+    fd_combine(A, 3 * vs + e, o3, q2, fma(C.ko, s2.ko, PMUL(P, C.r12, sp.d[1])), C.gdt, C.ddt);
+    q3 = S.val(4);
+    s3 = fd_stencil<4>(S, 4);
+    div = PADD(P, div, s3.d[2]);
+  }
+  const FdOld o0 = fd_old(A, e);
+  {
+    const auto S = stage(0);
+    fd_combine(A, 4 * vs + e, o4, q3, fma(C.ko, s3.ko, PMUL(P, C.r12, sp.d[2])), C.gdt, C.ddt);
+    fd_combine(A, vs + e, o1, Pi, fma(C.ko, sp.ko, fma(PMUL(P, PMUL(P, c, c), C.r12), div, PMUL(P, -P.damp, Pi))), C.gdt, C.ddt);
+    fd_combine(A, e, o0, S.val(0), fma(C.ko, fd_stencil<0>(S, 0).ko, Pi), C.gdt, C.ddt);
+  }
   if (A.lam_out) lam_thread = fmax(lam_thread, c);
 }
 
-template <class PDE, bool TMA>
+// Systems of at most five variables.  NB: boxes of the ring (the TMA-staged variants of the wave
+// system bring all five variables in one dense buffer instead).
+template <class PDE, bool TMA, int NB>
 __device__ void fd_tile_generic(const FdArgs& A, const FdWork& w, double* smem, uint64_t* bars, double& lam_thread) {
   static_assert(PDE::N <= GV, "generic FD path stages one group of at most five variables");
+  constexpr int N = PDE::N;
+  constexpr bool WAVE = std::is_same<PDE, PdeWave>::value;
+  static_assert(!TMA || WAVE, "TMA staging is compiled for the wave system");
   const dh_patch& pt = A.patches[w.patch];
   const int p = pt.p;
   const int t = threadIdx.x;
   const int lx = t % FTX, ly = (t / FTX) % FTY, lz = t / (FTX * FTY);
   const int64_t e = pt.offset + ((int64_t)(w.z0 + lz) * p + (w.y0 + ly)) * p + (w.x0 + lx);
-  if (TMA) {
+  __shared__ FdScalars C;
+  if constexpr (TMA) {
     if (t == 0) tma_issue(A, w, p, smem, &bars[0], 0);
+    fd_scalars(A, pt.dx, &C);
     if (!tma_wait_all(A, &bars[0], 0)) return;
-    if constexpr (std::is_same<PDE, PdeWave>::value) fd_voxel_wave(A, TmaAcc{smem, lx, ly, lz}, e, pt.dx, lam_thread);
-    else fd_voxel_generic<PDE>(A, TmaAcc{smem, lx, ly, lz}, e, pt.dx, lam_thread);
+    fd_voxel_wave(A, [&](int) { return TmaAcc{smem, lx, ly, lz}; }, e, C, lam_thread);
   } else {
-    fd_stage_vars(A, smem, w, p, 0, PDE::N);
-    __syncthreads();
-    if constexpr (std::is_same<PDE, PdeWave>::value) fd_voxel_wave(A, BoxAcc{smem, fd_box(lx, ly, lz)}, e, pt.dx, lam_thread);
-    else fd_voxel_generic<PDE>(A, BoxAcc{smem, fd_box(lx, ly, lz)}, e, pt.dx, lam_thread);
+    FdRing<NB> R(A, w, p, smem);
+    auto var = [](int i) { return i >= N ? -1 : (WAVE ? (i + 1) % N : i); };  // order of the variables
+#pragma unroll
+    for (int i = 0; i < NB - 1; ++i) R.issue(var(i), i);
+    fd_scalars(A, pt.dx, &C);
+    auto stage = [&](int i) {  // i-th variable of the order
+      R.wait();
+      R.issue(var(i + NB - 1), (i + NB - 1) % NB);
+      return R.acc(i % NB);
+    };
+    if constexpr (WAVE) {
+      fd_voxel_wave(A, [&](int v) { return stage(v == 0 ? 4 : v - 1); }, e, C, lam_thread);
+    } else {
+      double q[N + PDE::M], ko[N], dq[3][N];
+#pragma unroll
+      for (int v = 0; v < PDE::M; ++v) q[N + v] = __ldg(A.mat + (int64_t)v * A.vs + e);
+#pragma unroll
+      for (int v = 0; v < N; ++v) {
+        const BoxAcc S = stage(v);
+        q[v] = S.val(v);
+        const Stencil s = fd_stencil<7>(S, v);
+        ko[v] = s.ko;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) dq[d][v] = PDE::needs_grad(d, v) ? PMUL(A.P, s.d[d], C.r12) : 0.0;
+      }
+      fd_finish_generic<PDE>(A, q, ko, dq, e, C, lam_thread);
+    }
   }
 }
 
@@ -404,116 +554,126 @@ struct Gw59State {
   double alr, bxr, byr, bzr;  // alpha and beta times 1/(12 dx): the field derivatives stay unscaled
 };
 
-template <class Acc>
-__device__ __forceinline__ void gw59_lapse_shift(const FdArgs& A, const Acc& S, int64_t e, double r12, double ko,
-                                                 Gw59State& G) {
-  const DevParams& P = A.P;
-  G.al = S.val(0); G.bx = S.val(1); G.by = S.val(2); G.bz = S.val(3);
-  G.alr = PMUL(P, G.al, r12); G.bxr = PMUL(P, G.bx, r12); G.byr = PMUL(P, G.by, r12); G.bzr = PMUL(P, G.bz, r12);
-  G.dal0 = acc_d1<0>(P, S, 0, r12);
-  G.dal1 = acc_d1<1>(P, S, 0, r12);
-  G.dal2 = acc_d1<2>(P, S, 0, r12);
-#pragma unroll
-  for (int v = 0; v < 4; ++v) G.ko_ab[v] = PMUL(P, ko, acc_ko3(P, S, v));
-  // phi_b Pi_b at this voxel for the source coupling
-#pragma unroll
-  for (int bb = 0; bb < 11; ++bb)
-    G.u[bb] = PMUL(P, __ldg(A.qs + (int64_t)(5 * bb) * A.vs + e), __ldg(A.qs + (int64_t)(5 * bb + 1) * A.vs + e));
-  G.sumPi2 = 0.0; G.bs0 = 0.0; G.bs1 = 0.0; G.bs2 = 0.0;
-}
-
-template <class Acc>
-__device__ __forceinline__ void gw59_field(const FdArgs& A, const Acc& S, int a, int64_t e, double r12, double ko,
-                                           double gdt, double ddt, Gw59State& G) {
-  const DevParams& P = A.P;
-  const int64_t vs = A.vs;
-  const double al = G.al, bx = G.bx, by = G.by, bz = G.bz;
-  const double phi = S.val(0), Pi = S.val(1), px = S.val(2), py = S.val(3), pz = S.val(4);
-  // unscaled derivatives (the 1/(12 dx) sits in alr, bxr, byr, bzr)
-  const double dPi0 = acc_raw<0>(P, S, 1), dPi1 = acc_raw<1>(P, S, 1), dPi2 = acc_raw<2>(P, S, 1);
-  // coupling sum_b C_ab phi_b Pi_b
-  double cs = PMUL(P, P.C[11 * a], G.u[0]);
-#pragma unroll
-  for (int bb = 1; bb < 11; ++bb) cs = fma(P.C[11 * a + bb], G.u[bb], cs);
-  // phi: alpha Pi + beta . psi
-  const double Lphi = fma(al, Pi, fma(bx, px, fma(by, py, PMUL(P, bz, pz))));
-  // Pi: alpha div psi + beta . grad Pi + alpha cs
-  const double dpx0 = acc_raw<0>(P, S, 2), dpx1 = acc_raw<1>(P, S, 2), dpx2 = acc_raw<2>(P, S, 2);
-  const double dpy0 = acc_raw<0>(P, S, 3), dpy1 = acc_raw<1>(P, S, 3), dpy2 = acc_raw<2>(P, S, 3);
-  const double dpz0 = acc_raw<0>(P, S, 4), dpz1 = acc_raw<1>(P, S, 4), dpz2 = acc_raw<2>(P, S, 4);
-  const double alr = G.alr, bxr = G.bxr, byr = G.byr, bzr = G.bzr;
-  const double LPi = fma(alr, PADD(P, PADD(P, dpx0, dpy1), dpz2), fma(bxr, dPi0, fma(byr, dPi1, fma(bzr, dPi2, PMUL(P, al, cs)))));
-  // psi_i: alpha d_i Pi + Pi d_i alpha + beta . grad psi_i
-  const double Lpx = fma(alr, dPi0, fma(Pi, G.dal0, fma(bxr, dpx0, fma(byr, dpx1, PMUL(P, bzr, dpx2)))));
-  const double Lpy = fma(alr, dPi1, fma(Pi, G.dal1, fma(bxr, dpy0, fma(byr, dpy1, PMUL(P, bzr, dpy2)))));
-  const double Lpz = fma(alr, dPi2, fma(Pi, G.dal2, fma(bxr, dpz0, fma(byr, dpz1, PMUL(P, bzr, dpz2)))));
-  G.sumPi2 = fma(Pi, Pi, G.sumPi2);
-  G.bs0 = fma(px, Pi, G.bs0);
-  G.bs1 = fma(py, Pi, G.bs1);
-  G.bs2 = fma(pz, Pi, G.bs2);
-  const int64_t eb = (int64_t)(5 * a) * vs + e;
-  fd_combine(A, eb, phi, fma(ko, acc_ko3(P, S, 0), Lphi), gdt, ddt);
-  fd_combine(A, eb + vs, Pi, fma(ko, acc_ko3(P, S, 1), LPi), gdt, ddt);
-  fd_combine(A, eb + 2 * vs, px, fma(ko, acc_ko3(P, S, 2), Lpx), gdt, ddt);
-  fd_combine(A, eb + 3 * vs, py, fma(ko, acc_ko3(P, S, 3), Lpy), gdt, ddt);
-  fd_combine(A, eb + 4 * vs, pz, fma(ko, acc_ko3(P, S, 4), Lpz), gdt, ddt);
-}
-
 __device__ __forceinline__ void gw59_finish(const FdArgs& A, int64_t e, double gdt, double ddt, const Gw59State& G,
                                             double& lam_thread) {
   const DevParams& P = A.P;
   const int64_t vs = A.vs;
   const double Lal = fma(PMUL(P, -P.kappa, PMUL(P, G.al, G.al)), G.sumPi2, G.ko_ab[0]);
-  const double ra = fd_combine(A, 55 * vs + e, G.al, Lal, gdt, ddt);
-  const double r0 = fd_combine(A, 56 * vs + e, G.bx, fma(0.75, G.bs0, G.ko_ab[1]), gdt, ddt);
-  const double r1 = fd_combine(A, 57 * vs + e, G.by, fma(0.75, G.bs1, G.ko_ab[2]), gdt, ddt);
-  const double r2 = fd_combine(A, 58 * vs + e, G.bz, fma(0.75, G.bs2, G.ko_ab[3]), gdt, ddt);
+  const double ra = fd_combine(A, 55 * vs + e, fd_old(A, 55 * vs + e), G.al, Lal, gdt, ddt);
+  const double r0 = fd_combine(A, 56 * vs + e, fd_old(A, 56 * vs + e), G.bx, fma(0.75, G.bs0, G.ko_ab[1]), gdt, ddt);
+  const double r1 = fd_combine(A, 57 * vs + e, fd_old(A, 57 * vs + e), G.by, fma(0.75, G.bs1, G.ko_ab[2]), gdt, ddt);
+  const double r2 = fd_combine(A, 58 * vs + e, fd_old(A, 58 * vs + e), G.bz, fma(0.75, G.bs2, G.ko_ab[3]), gdt, ddt);
   if (A.lam_out) lam_thread = fmax(lam_thread, PADD(P, ra, fmax(fmax(fabs(r0), fabs(r1)), fabs(r2))));
 }
 
-template <bool TMA>
-__device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, uint64_t* bars, double& lam_thread) {
+// Variables in the order lapse, shift x, y, z, then per field Pi, psi_x, psi_y, psi_z, phi: each is
+// read from its box once, while the next ones stream in.
+template <int NB>
+__device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, double& lam_thread) {
+  const DevParams& P = A.P;
+  const int64_t vs = A.vs;
   const dh_patch& pt = A.patches[w.patch];
   const int p = pt.p;
-  const int t = threadIdx.x;
-  const int lx = t % FTX, ly = (t / FTX) % FTY, lz = t / (FTX * FTY);
-  const int64_t e = pt.offset + ((int64_t)(w.z0 + lz) * p + (w.y0 + ly)) * p + (w.x0 + lx);
-  const double dx = pt.dx;
-  const double r12 = 1.0 / (12.0 * dx);
-  const double ko = A.sigma / (64.0 * dx);
-  const double dt = *A.dt_dev;
-  const double gdt = A.g * dt, ddt = A.d * dt;
+  __shared__ FdScalars C;
+  FdRing<NB> R(A, w, p, smem);
+  const int64_t e = R.e[0];
+  auto var = [](int i) {  // i-th variable of the order
+    if (i < 4) return 55 + i;
+    if (i >= 59) return -1;
+    const int a = (i - 4) / 5, j = (i - 4) - 5 * a;
+    return 5 * a + (j == 4 ? 0 : j + 1);
+  };
+#pragma unroll
+  for (int i = 0; i < NB - 1; ++i) R.issue(var(i), i);
+  fd_scalars(A, pt.dx, &C);
+  int next = NB - 1, buf = 0;  // next variable of the order to issue, box of the current one
+  auto stage = [&]() {
+    R.wait();
+    R.issue(var(next++), buf == 0 ? NB - 1 : buf - 1);
+    const BoxAcc S = R.acc(buf);
+    buf = buf == NB - 1 ? 0 : buf + 1;
+    return S;
+  };
   Gw59State G;
-  if (TMA) {
-    // groups: 0 = lapse/shift (variables 55..59, 59 out of range reads as 0), 1..11 = fields 0..10
-    if (t == 0) tma_issue(A, w, p, smem, &bars[0], 55);
+  // phi_b Pi_b at this voxel for the source coupling
+#pragma unroll
+  for (int bb = 0; bb < 11; ++bb)
+    G.u[bb] = PMUL(P, __ldg(A.qs + (int64_t)(5 * bb) * vs + e), __ldg(A.qs + (int64_t)(5 * bb + 1) * vs + e));
+  G.sumPi2 = 0.0; G.bs0 = 0.0; G.bs1 = 0.0; G.bs2 = 0.0;
+  {
+    const BoxAcc S = stage();
+    const double r12 = C.r12;
+    G.al = S.val(0);
+    const Stencil s = fd_stencil<7>(S, 0);
+    G.dal0 = PMUL(P, s.d[0], r12);
+    G.dal1 = PMUL(P, s.d[1], r12);
+    G.dal2 = PMUL(P, s.d[2], r12);
+    G.ko_ab[0] = PMUL(P, C.ko, s.ko);
+    G.alr = PMUL(P, G.al, r12);
+  }
+#pragma unroll
+  for (int v = 1; v < 4; ++v) {
+    const BoxAcc S = stage();
+    const double b = S.val(0);
+    (v == 1 ? G.bx : v == 2 ? G.by : G.bz) = b;
+    (v == 1 ? G.bxr : v == 2 ? G.byr : G.bzr) = PMUL(P, b, C.r12);
+    G.ko_ab[v] = PMUL(P, C.ko, fd_stencil<0>(S, 0).ko);
+  }
+  const double ko = C.ko, gdt = C.gdt, ddt = C.ddt;
+  const double al = G.al, bx = G.bx, by = G.by, bz = G.bz, alr = G.alr, bxr = G.bxr, byr = G.byr, bzr = G.bzr;
+  double phi = 0.0, Lphi = 0.0;  // the field before: its phi and L_phi, updated in the next field's first step
+  FdOld op{0.0, 0.0};
 #pragma unroll 1
-    for (int gi = 0; gi < 12; ++gi) {
-      const int b = gi & 1;
-      if (gi + 1 < 12 && t == 0) tma_issue(A, w, p, smem + (b ^ 1) * TBUF, &bars[b ^ 1], 5 * gi);
-      if (!tma_wait_all(A, &bars[b], (gi >> 1) & 1)) {
-        // abandon the tile; the copy issued into the other buffer may still be in flight
-        if (gi + 1 < 12) mbar_wait(&bars[b ^ 1], ((gi + 1) >> 1) & 1);
-        return;
-      }
-      const TmaAcc S{smem + b * TBUF, lx, ly, lz};
-      if (gi == 0) gw59_lapse_shift(A, S, e, r12, ko, G);
-      else gw59_field(A, S, gi - 1, e, r12, ko, gdt, ddt, G);
-      __syncthreads();  // buffer b is free for the copy issued in the next iteration
+  for (int a = 0; a < 11; ++a) {
+    const int64_t eb = (int64_t)(5 * a) * vs + e;
+    // Pi: alpha div psi + beta . grad Pi + alpha cs;  psi_i: alpha d_i Pi + Pi d_i alpha + beta . grad psi_i
+    // (unscaled derivatives: the 1/(12 dx) sits in alr, bxr, byr, bzr).  A variable's update stands
+    // after the staging of the next one, so that its FP64 operations can be issued among the
+    // integer operations of the next stencil.
+    double Pi, LPi, div = 0.0, ps = 0.0;
+    Stencil sP, s;
+    FdOld oP = fd_old(A, eb + vs), o;
+    {
+      const BoxAcc S = stage();
+      if (a > 0) fd_combine(A, eb - 5 * vs, op, phi, Lphi, gdt, ddt);
+      Pi = S.val(0);
+      sP = fd_stencil<7>(S, 0);
     }
-  } else {
-    const BoxAcc S{smem, fd_box(lx, ly, lz)};
-    fd_stage_vars(A, smem, w, p, 55, 4);
-    __syncthreads();
-    gw59_lapse_shift(A, S, e, r12, ko, G);
-#pragma unroll 1
-    for (int a = 0; a < 11; ++a) {
-      __syncthreads();  // previous group's box reads are done
-      fd_stage_vars(A, smem, w, p, 5 * a, 5);
-      __syncthreads();
-      gw59_field(A, S, a, e, r12, ko, gdt, ddt, G);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // psi_x, psi_y, psi_z, phi
+      const FdOld on = fd_old(A, eb + (i < 3 ? 2 + i : 0) * vs);
+      const BoxAcc S = stage();
+      if (i == 0) {
+        Lphi = PMUL(P, al, Pi);
+        G.sumPi2 = fma(Pi, Pi, G.sumPi2);
+        // coupling sum_b C_ab phi_b Pi_b
+        double cs = PMUL(P, P.C[11 * a], G.u[0]);
+#pragma unroll
+        for (int bb = 1; bb < 11; ++bb) cs = fma(P.C[11 * a + bb], G.u[bb], cs);
+        LPi = fma(ko, sP.ko, fma(bxr, sP.d[0], fma(byr, sP.d[1], fma(bzr, sP.d[2], PMUL(P, al, cs)))));
+      } else {
+        const int j = i - 1;
+        div = j == 0 ? s.d[0] : PADD(P, div, s.d[j]);
+        Lphi = fma(j == 0 ? bx : j == 1 ? by : bz, ps, Lphi);
+        double& bs = j == 0 ? G.bs0 : j == 1 ? G.bs1 : G.bs2;
+        bs = fma(ps, Pi, bs);
+        const double L = fma(alr, sP.d[j], fma(Pi, j == 0 ? G.dal0 : j == 1 ? G.dal1 : G.dal2,
+                                               fma(bxr, s.d[0], fma(byr, s.d[1], PMUL(P, bzr, s.d[2])))));
+        fd_combine(A, eb + (2 + j) * vs, o, ps, fma(ko, s.ko, L), gdt, ddt);
+      }
+      if (i == 3) {
+        fd_combine(A, eb + vs, oP, Pi, fma(alr, div, LPi), gdt, ddt);
+        phi = S.val(0);
+        op = on;
+        Lphi = fma(ko, fd_stencil<0>(S, 0).ko, Lphi);
+      } else {
+        ps = S.val(0);
+        o = on;
+        s = fd_stencil<7>(S, 0);
+      }
     }
   }
+  fd_combine(A, 50 * vs + e, op, phi, Lphi, gdt, ddt);
   gw59_finish(A, e, gdt, ddt, G, lam_thread);
 }
 
@@ -547,44 +707,49 @@ __device__ void fd_publish_lambda(double lam, double* lam_out, unsigned long lon
 }
 
 // Kernel variants (chosen per plan by the autotuner):
-//   VAR bit 1: at most 128 registers so that two CTAs fit on an SM;
-//   VAR bit 2: TMA staging (double-buffered groups) instead of plain loads;
-//   VAR bit 3 / bit 4: register caps for three / four CTAs per SM (80 / 64
-//              registers; with TMA staging the single group buffer of the
-//              generic path, 43.6 KB, lets that many CTAs share an SM).
-template <int VAR>
+//   VAR bit 1: at most 128 registers so that two CTAs fit on an SM, five boxes (else 80 registers
+//              and four boxes for three CTAs); GW59 has the first form only;
+//   VAR bit 2: TMA staging of all variables in one dense buffer instead of the ring (wave system);
+//   VAR bit 3 / bit 4: with TMA staging, register caps for three / four CTAs per SM (80 / 64
+//              registers; the buffer takes 43.6 KB).
+template <class PDE, int VAR>
 constexpr int fd_min_blocks() {
-  return (VAR & 16) ? 4 : (VAR & 8) ? 3 : (VAR & 2) ? 2 : 1;
+  return (VAR & 16) ? 4 : (VAR & 8) ? 3 : (VAR & 2) ? 2 : (VAR & 4) ? 1 : 3;
+}
+// Boxes of the ring: as many as fit beside the other CTAs of the SM, at most the variables.
+template <class PDE, int VAR>
+constexpr int fd_ring() {
+  return PDE::N == 59 ? 6 : (VAR & 2) ? 5 : 4;
 }
 
 template <class PDE, int VAR>
-__global__ void __launch_bounds__(FNT, fd_min_blocks<VAR>()) k_fd_stage(const __grid_constant__ FdArgs A) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2];
+__global__ void __launch_bounds__(FNT, (fd_min_blocks<PDE, VAR>())) k_fd_stage(const __grid_constant__ FdArgs A) {
+  extern __shared__ __align__(128) double fd_smem[];
+  __shared__ __align__(8) uint64_t bars[1];
   constexpr bool TMA = (VAR & 4) != 0;
-  // TMA destinations start on a 128-byte boundary (the launch adds 128 bytes of slack)
-  double* smem = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
-  if (TMA) {
+  constexpr int NB = fd_ring<PDE, VAR>();
+  const FdWork w = A.work[blockIdx.x];
+  double lam = 0.0;
+  if constexpr (TMA) {
+    // TMA destinations start on a 128-byte boundary (the launch adds 128 bytes of slack)
+    double* smem = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(fd_smem) + 127) & ~(uintptr_t)127);
     if (threadIdx.x == 0) {
       mbar_init(&bars[0], 1);
-      mbar_init(&bars[1], 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    fd_tile_generic<PDE, true, NB>(A, w, smem, bars, lam);
+  } else if constexpr (PDE::N == 59) {
+    fd_tile_gw59<NB>(A, w, fd_smem, lam);
+  } else {
+    fd_tile_generic<PDE, false, NB>(A, w, fd_smem, bars, lam);
   }
-  const FdWork w = A.work[blockIdx.x];
-  double lam = 0.0;
-  if constexpr (PDE::N == 59) fd_tile_gw59<TMA>(A, w, smem, bars, lam);
-  else fd_tile_generic<PDE, TMA>(A, w, smem, bars, lam);
   if (A.lam_out) fd_publish_lambda(lam, A.lam_out, A.red);
 }
 
 template <class PDE, int VAR>
 static dh_status fd_launch_var(dh_plan* plan, const FdArgs& A, cudaStream_t stream) {
-  constexpr bool TMA = (VAR & 4) != 0;
-  constexpr int NB = PDE::N == 59 ? 5 : PDE::N;
-  // TMA: GW59 double-buffers its field groups, the generic path stages one group
-  const size_t smem = (TMA ? (PDE::N == 59 ? 2 : 1) * (size_t)TBYTES : sizeof(double) * NB * FBOX) + 128;
+  constexpr size_t smem = (VAR & 4) ? (size_t)TBYTES + 128 : sizeof(double) * fd_ring<PDE, VAR>() * FBOX;
   static int configured_device = -1;
   if (configured_device != plan->device) {
     cudaError_t e = cudaFuncSetAttribute(k_fd_stage<PDE, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -595,17 +760,23 @@ static dh_status fd_launch_var(dh_plan* plan, const FdArgs& A, cudaStream_t stre
   return cuda_error(cudaGetLastError(), "k_fd_stage launch");
 }
 
+// The TMA-staged variants are compiled for the wave system; the others run the ring for them.
 template <class PDE>
 static dh_status fd_launch(dh_plan* plan, const FdArgs& A, cudaStream_t stream) {
-  if constexpr (PDE::N != 59) {
-    if (plan->fd_var == 12) return fd_launch_var<PDE, 12>(plan, A, stream);
-    if (plan->fd_var == 20) return fd_launch_var<PDE, 20>(plan, A, stream);
+  if constexpr (std::is_same<PDE, PdeWave>::value) {
+    switch (plan->fd_var) {
+      case 4: return fd_launch_var<PDE, 4>(plan, A, stream);
+      case 6: return fd_launch_var<PDE, 6>(plan, A, stream);
+      case 12: return fd_launch_var<PDE, 12>(plan, A, stream);
+      case 20: return fd_launch_var<PDE, 20>(plan, A, stream);
+      default: break;
+    }
   }
-  switch (plan->fd_var & 6) {
-    case 0: return fd_launch_var<PDE, 0>(plan, A, stream);
-    case 2: return fd_launch_var<PDE, 2>(plan, A, stream);
-    case 4: return fd_launch_var<PDE, 4>(plan, A, stream);
-    default: return fd_launch_var<PDE, 6>(plan, A, stream);
+  if constexpr (PDE::N == 59) {
+    return fd_launch_var<PDE, 2>(plan, A, stream);
+  } else {
+    if (plan->fd_var & 2) return fd_launch_var<PDE, 2>(plan, A, stream);
+    return fd_launch_var<PDE, 0>(plan, A, stream);
   }
 }
 
@@ -657,14 +828,18 @@ static dh_status encode_maps(dh_plan* plan, const double* qs, FdArgs& A) {
 
 dh_status launch_fd_stage(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc,
                           const double* mat, const double* dt_dev, double a, double b, double g, double d,
-                          double sigma, double* lam_out, cudaStream_t stream) {
+                          double sigma, double* lam_out, cudaStream_t stream, const double* acc_in,
+                          double* acc_copy) {
   FdArgs A;
   std::memset(&A.maps, 0, sizeof(A.maps));
   A.patches = plan->d_patches;
   A.work = plan->d_fdwork;
   A.lvl = plan->d_lvl;
   A.qs = qs; A.q0 = q0; A.out = out; A.acc = acc; A.mat = mat; A.dt_dev = dt_dev;
+  A.acc_in = acc_in ? acc_in : acc;
+  A.acc_copy = acc_copy;
   A.a = a; A.b = b; A.g = g; A.d = d; A.sigma = sigma;
+  A.a1 = a == 1.0; A.b1 = b == 1.0; A.b0 = b == 0.0;
   A.lam_out = lam_out;
   A.red = plan->d_red;
   A.err = reinterpret_cast<unsigned int*>(plan->d_red + 2);

@@ -198,9 +198,17 @@ dh_status aoas_move(dh_plan* plan, bool gather, const double* const* blocks, int
 dh_status rk_steps(dh_plan* plan, int scheme, int rk, int n_steps, double* q, double* u1, double* u2, double* acc,
                    const double* mat, double* dt, double* lam, double cfl, double sigma, cudaStream_t s);
 
+// acc_in: acc = acc_in + d dt L (NULL: acc itself); acc_copy: NULL, or a second array that
+// receives the new acc (it may be an array the stage does not read).
 dh_status launch_fd_stage(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc,
                           const double* mat, const double* dt_dev, double a, double b, double g, double d,
-                          double sigma, double* lam_out, cudaStream_t stream);
+                          double sigma, double* lam_out, cudaStream_t stream, const double* acc_in = nullptr,
+                          double* acc_copy = nullptr);
+
+// patch_update_fd_ko with the accumulation's source and copy of launch_fd_stage.
+dh_status fd_stage(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc, const double* mat,
+                   const double* dt_dev, double a, double b, double g, double d, double sigma_ko, double* lam_out_dev,
+                   cudaStream_t stream, const double* acc_in, double* acc_copy);
 
 dh_status launch_fv2_stage(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc,
                            const double* mat, const double* dt_dev, double a, double b, double g, double d,

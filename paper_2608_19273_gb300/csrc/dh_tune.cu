@@ -17,9 +17,8 @@
 //               column plane and its ring strips into a double-buffered shared ring
 //   second-order FV stage: z-march of whole patches or in chunks of <= 16 planes, or the 8x8x4
 //             tile kernel;
-//   FD stage: register cap (1 or 2 CTAs per SM) x staging (plain loads or TMA);
-//             with TMA staging of one group (systems of <= 5 variables) also
-//             caps for 3 and 4 CTAs per SM
+//   FD stage: register cap (3 or 2 CTAs per SM) x staging (asynchronous copies or TMA);
+//             with TMA staging (systems of <= 5 variables) also caps for 3 and 4 CTAs per SM
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
