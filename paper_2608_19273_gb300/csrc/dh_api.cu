@@ -324,6 +324,25 @@ static dh_status check_plan(const dh_plan* plan) {
   return DH_OK;
 }
 
+dh_status fd_stage(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc, const double* mat,
+                   const double* dt_dev, double a, double b, double g, double d, double sigma_ko, double* lam_out_dev,
+                   cudaStream_t stream, const double* acc_in, double* acc_copy) {
+  dh_status st = check_plan(plan);
+  if (st != DH_OK) return st;
+  if (plan->fv_generic) { set_error("patch_update_fd_ko: needs patch sizes that are multiples of 8"); return DH_EUNSUPPORTED; }
+  if (!qs || !dt_dev) { set_error("patch_update_fd_ko: qs and dt_dev are required"); return DH_EINVAL; }
+  if (!out && !acc) { set_error("patch_update_fd_ko: nothing to write (out and acc are NULL)"); return DH_EINVAL; }
+  if (plan->nm > 0 && !mat) { set_error("patch_update_fd_ko: PDE needs the material arena"); return DH_EINVAL; }
+  if (!q0 && a != 0.0) { set_error("patch_update_fd_ko: q0 is NULL but a != 0"); return DH_EINVAL; }
+  if (out == qs || acc == qs || (out && out == acc)) { set_error("patch_update_fd_ko: out/acc must not alias qs or each other"); return DH_EINVAL; }
+  if (plan->halo < 3) { set_error("patch_update_fd_ko: the plan needs halo >= 3 (it has %d)", plan->halo); return DH_EINVAL; }
+  if (plan->coupled) { set_error("patch_update_fd_ko: coupled refinement levels are supported by patch_update_fv only"); return DH_EUNSUPPORTED; }
+  if (plan->dim != 3) { set_error("patch_update_fd_ko: 3D only"); return DH_EUNSUPPORTED; }
+  if (!(sigma_ko >= 0.0)) { set_error("patch_update_fd_ko: sigma must be >= 0"); return DH_EINVAL; }
+  return launch_fd_stage(plan, qs, q0, out, acc, mat, dt_dev, a, b, g, d, sigma_ko, lam_out_dev, stream,
+                         acc_in, acc_copy);
+}
+
 }  // namespace dh
 
 using namespace dh;
@@ -617,19 +636,8 @@ dh_status patch_update_fv(dh_plan* plan, const double* qs, const double* q0, dou
 dh_status patch_update_fd_ko(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc,
                              const double* mat, const double* dt_dev, double a, double b, double g, double d,
                              double sigma_ko, double* lam_out_dev, void* stream) {
-  dh_status st = check_plan(plan);
-  if (st != DH_OK) return st;
-  if (plan->fv_generic) { set_error("patch_update_fd_ko: needs patch sizes that are multiples of 8"); return DH_EUNSUPPORTED; }
-  if (!qs || !dt_dev) { set_error("patch_update_fd_ko: qs and dt_dev are required"); return DH_EINVAL; }
-  if (!out && !acc) { set_error("patch_update_fd_ko: nothing to write (out and acc are NULL)"); return DH_EINVAL; }
-  if (plan->nm > 0 && !mat) { set_error("patch_update_fd_ko: PDE needs the material arena"); return DH_EINVAL; }
-  if (!q0 && a != 0.0) { set_error("patch_update_fd_ko: q0 is NULL but a != 0"); return DH_EINVAL; }
-  if (out == qs || acc == qs || (out && out == acc)) { set_error("patch_update_fd_ko: out/acc must not alias qs or each other"); return DH_EINVAL; }
-  if (plan->halo < 3) { set_error("patch_update_fd_ko: the plan needs halo >= 3 (it has %d)", plan->halo); return DH_EINVAL; }
-  if (plan->coupled) { set_error("patch_update_fd_ko: coupled refinement levels are supported by patch_update_fv only"); return DH_EUNSUPPORTED; }
-  if (plan->dim != 3) { set_error("patch_update_fd_ko: 3D only"); return DH_EUNSUPPORTED; }
-  if (!(sigma_ko >= 0.0)) { set_error("patch_update_fd_ko: sigma must be >= 0"); return DH_EINVAL; }
-  return launch_fd_stage(plan, qs, q0, out, acc, mat, dt_dev, a, b, g, d, sigma_ko, lam_out_dev, (cudaStream_t)stream);
+  return fd_stage(plan, qs, q0, out, acc, mat, dt_dev, a, b, g, d, sigma_ko, lam_out_dev, (cudaStream_t)stream, nullptr,
+                  nullptr);
 }
 
 dh_status patch_update_fv_muscl(dh_plan* plan, const double* qs, const double* q0, double* out, double* acc,
