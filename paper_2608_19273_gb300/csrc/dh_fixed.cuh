@@ -51,4 +51,43 @@ __device__ __forceinline__ double fx_value(long long t, int e) {
   return t == 0 ? 0.0 : __hiloint2double(hi, __double2loint(f));
 }
 
+// p[0] + .. + p[NP-1] - m[0] - .. - m[NM-1], with NP + NM <= 24 (five bits above the 53 + 5 of a
+// term): about 13 integer instructions per term and one conversion, instead of NP + NM - 1 FP64
+// additions.  With NP = NM and p[i] = m[i] the sum is exactly 0 in either form.
+template <int NP, int NM>
+__device__ __forceinline__ double fx_sum(const double (&p)[NP], const double (&m)[NM]) {
+  static_assert(NP + NM <= 24 && NM <= NP, "room for the terms");
+  constexpr int SH = 5;
+  int e = 0;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) e = max(e, fx_exp(p[i]));
+#pragma unroll
+  for (int i = 0; i < NM; ++i) e = max(e, fx_exp(m[i]));
+  if (!fx_ok(e)) {
+    long long any = 0;  // zeros (a quantity at rest) are the usual case here
+#pragma unroll
+    for (int i = 0; i < NP; ++i) any |= __double_as_longlong(p[i]);
+#pragma unroll
+    for (int i = 0; i < NM; ++i) any |= __double_as_longlong(m[i]);
+    if ((any & 0x7fffffffffffffffll) == 0) return 0.0;
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) s += i < NM ? p[i] - m[i < NM ? i : 0] : p[i];
+    return s;
+  }
+  long long t = 0;
+  int neg = 0;  // the unit that each complemented term lacks: sums of terms that fit are exact
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    t += fx_align<SH>(p[i], e);
+    neg -= __double2hiint(p[i]) >> 31;
+  }
+#pragma unroll
+  for (int i = 0; i < NM; ++i) {
+    t -= fx_align<SH>(m[i], e);
+    neg += __double2hiint(m[i]) >> 31;
+  }
+  return fx_value<SH>(t + neg, e);
+}
+
 }  // namespace dh

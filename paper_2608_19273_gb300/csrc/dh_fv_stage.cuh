@@ -22,16 +22,26 @@
 //   * A CTA owns a (TX x TY) column of one patch -- 16x16 or 32x8 -- (or four 8x8
 //     columns of up to four patches) and marches it through the z-planes of the
 //     patch; in the persistent form a CTA takes tile after tile from a queue.
-//   * Per voxel, the derived quantities W (one reciprocal, one square root for
-//     Euler), the three directional fluxes F_d and speeds lambda_d are computed
-//     exactly once.  x/y neighbours exchange them through shared memory; the
-//     z neighbour is the same thread one plane later (registers).
+//   * Per voxel, the derived quantities W (one reciprocal, one square root for Euler), the
+//     three speeds and the cell terms of the fluxes (pressure, cross_term) are computed exactly
+//     once.  x/y neighbours exchange them through shared memory; the z neighbour is the same
+//     thread one plane later (registers).
 //   * The ring of halo voxels around the column (neighbour patches or the
 //     rest of the same patch) is computed by the first 2(TX+TY)G threads;
 //     ring voxels only need the one direction that crosses into the column.
-//   * Every face flux is computed once: each voxel thread computes its -x and
+//   * Every face value is computed once: each voxel thread computes its -x and
 //     -y faces, the +x/+y boundary faces are computed by ring threads; the
 //     factor 1/2 of the Rusanov average is folded into the final -1/(2dx).
+//     A face value is Q_L (u_L + s) + Q_R (u_R - s) (rusanov): two operations per
+//     quantity and no flux per cell (it was 12 for the fluxes of a voxel and 3 per quantity and face).
+//   * The sum over a voxel's faces and cell terms is formed in fixed point on the integer pipe
+//     (fx_sum): 6 to 13 terms per quantity cost one conversion, not as many FP64 additions.
+//   Euler in 3D issues 80 FP64 instructions a voxel and stage (117 before these two), with the pipe
+//   75-80% busy: 10.5 M voxels of the 8^3/16^3/32^3 mix, two SSP-RK3 steps, 15.2 -> 10.9 ms.  The pipe is still
+//   the bound; the integer one is a quarter busy.  Measured on the way: the two changes alone 12.0;
+//   the z face after the barrier (beside the sums) and the plane's loads before the in-plane
+//   faces 11.65; the earlier stages' sums and state loaded before the barrier 10.9.  24 warps an SM
+//   at 80 registers (spills): 12.9.
 //   * The maximum characteristic speed of the result is reduced with warp
 //     shuffles, then one atomicMax per CTA on the bit pattern (valid for
 //     non-negative doubles), and the last CTA publishes it (no spin waits).
@@ -40,6 +50,9 @@
 #include <algorithm>
 #include <type_traits>
 
+#include <utility>
+
+#include "dh_fixed.cuh"
 #include "dh_internal.cuh"
 #include "dh_pde.cuh"
 #include "dh_tma.cuh"
@@ -171,17 +184,14 @@ __device__ __forceinline__ void derive(const FvArgs& A, int64_t e, const double*
   }
 }
 
-// F_x and F_y of one voxel (F_z already formed in 3D): systems with a symmetric
-// flux share its off-diagonal products between directions.
-template <class PDE>
-__device__ __forceinline__ void flux_xy(const double* q, const double* W, const double* Fz, const DevParams& P,
-                                        double* Fx, double* Fy) {
-  if constexpr (PDE::SYM) {
-    PDE::flux_xy(q, W, Fz, P, Fx, Fy);
-  } else {
-    PDE::flux(0, q, W, P, Fx);
-    PDE::flux(1, q, W, P, Fy);
-  }
+// f(integral_constant<int, 0>), f(integral_constant<int, 1>), ..: a loop whose index is a constant.
+template <class F, int... I>
+__device__ __forceinline__ void for_seq(F f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void for_n(F f) {
+  for_seq(f, std::make_integer_sequence<int, N>{});
 }
 
 // Systems whose derived quantities are many (SRHD: eight) form all three
@@ -205,7 +215,12 @@ struct FvTile {
   // ring occupies warps 0 and 1, so the faces go to warp 2 (another SM
   // sub-partition: the extra FP64 work of a plane is spread over three of them)
   static constexpr int FT0 = (NR <= 64 && NT >= 96) ? 64 : 0;
-  static constexpr size_t SMEM_BASE = sizeof(double) * ((size_t)NV * NS + 2 * (size_t)N * NS + 2 * NS +
+  // cell terms (HYDRO systems: pressure and the x and y cross terms), read by the update of a plane
+  // while the next plane is published: interior slots once per plane parity, then the ring buffers
+  static constexpr bool HYDRO = PDE::HYDRO;
+  static constexpr int NX = HYDRO ? 3 : 0, NXS = 2 * NT + 2 * NR;
+  static constexpr int NU = HYDRO ? 4 : 2;  // per slot: u_x, u_y (HYDRO), lambda_x, lambda_y
+  static constexpr size_t SMEM_BASE = sizeof(double) * ((size_t)(NV + NU) * NS + (size_t)NX * NXS +
                                                         (size_t)NF * N * (FX + FY));
   // TMA staging (one column, 3D, no material): two plane buffers, each holding the interior
   // [N][TY][TX] and the ring strips -x, +x [N][TY][2] and -y, +y [N][TX] of one z-plane
@@ -220,16 +235,15 @@ struct FvTile {
   static_assert(NT == 256 || NT == 64, "tile classes use 256 threads, or 64 (one 8x8 column)");
 
   struct Smem {
-    double *Q, *Fx, *Fy, *Lx, *Ly, *Hx, *Hy, *Dx, *Dy;
+    double *Q, *U, *L, *X, *Hx, *Hy, *Dx, *Dy;  // U, L: x then y; X: pressure, cross x, cross y
     double* st[2];  // TMA plane buffers (128-byte aligned)
   };
   __device__ static Smem carve(double* s) {
     Smem S;
     S.Q = s; s += NV * NS;
-    S.Fx = s; s += N * NS;
-    S.Fy = s; s += N * NS;
-    S.Lx = s; s += NS;
-    S.Ly = s; s += NS;
+    S.U = s; if (HYDRO) s += 2 * NS;
+    S.L = s; s += 2 * NS;
+    S.X = s; s += NX * NXS;
     S.Hx = s; s += N * FX;
     S.Hy = s; s += N * FY;
     S.Dx = s; if (PDE::NCP) s += N * FX;
@@ -276,31 +290,59 @@ struct FvTile {
     else fvtma::load5(buf + ST_YP, &L[BY], x0, 0, z, A.lvl[pt.nbr[3]].y, 0, bar);
   }
 
-  // Face value F^' = (FL + FR) - s (QR - QL)  (twice the Rusanov flux) and,
-  // for non-conservative systems, D = B_d((QL+QR)/2)(QR - QL).
+  // Velocity along x or y of slot s (systems without one in W: the material velocity).
+  __device__ static double vel_at(const Smem& S, int d, int s) {
+    return HYDRO ? S.U[d * NS + s] : S.Q[(N + d) * NS + s];
+  }
+  // Two-sided part of twice the Rusanov flux (rusanov) of the face between slots Ls and Rs and, for
+  // non-conservative systems, D = B_d((QL+QR)/2)(QR - QL).
   __device__ static void face(const Smem& S, const DevParams& P, int d, int Ls, int Rs, double* H, double* D,
                               int fidx, int fstride) {
-    const double* F = d == 0 ? S.Fx : S.Fy;
-    const double* L = d == 0 ? S.Lx : S.Ly;
-    const double s = max_nn(L[Ls], L[Rs]);
-    double dq[N];
+    double qL[N], qR[N], h[N];
 #pragma unroll
-    for (int v = 0; v < N; ++v) {
-      const double qL = S.Q[v * NS + Ls], qR = S.Q[v * NS + Rs];
-      dq[v] = SUB(P, qR, qL);
-      double h;
-      if (PDE::FLUX) h = fma(-s, dq[v], ADD(P, F[v * NS + Ls], F[v * NS + Rs]));
-      else h = MUL(P, -s, dq[v]);
-      H[v * fstride + fidx] = h;
-    }
+    for (int v = 0; v < N; ++v) { qL[v] = S.Q[v * NS + Ls]; qR[v] = S.Q[v * NS + Rs]; }
+    rusanov<PDE>(P, qL, vel_at(S, d, Ls), S.L[d * NS + Ls], qR, vel_at(S, d, Rs), S.L[d * NS + Rs], h);
+#pragma unroll
+    for (int v = 0; v < N; ++v) H[v * fstride + fidx] = h[v];
     if (PDE::NCP) {
-      double qb[NV], Dv[N];
+      double qb[NV], dq[N], Dv[N];
+#pragma unroll
+      for (int v = 0; v < N; ++v) dq[v] = SUB(P, qR[v], qL[v]);
 #pragma unroll
       for (int v = 0; v < NV; ++v) qb[v] = MUL(P, 0.5, ADD(P, S.Q[v * NS + Ls], S.Q[v * NS + Rs]));
       PDE::ncp(d, qb, dq, P, Dv);
 #pragma unroll
       for (int v = 0; v < N; ++v) D[v * fstride + fidx] = Dv[v];
     }
+  }
+  // The same for the face between two cells of a column, z below z + 1.
+  __device__ static void face_z(const DevParams& P, const double* qL, double uL, double lL, const double* qR, double uR,
+                                double lR, double* H, double* D) {
+    rusanov<PDE>(P, qL, uL, lL, qR, uR, lR, H);
+    if (PDE::NCP) {
+      double qb[NV], dq[N];
+#pragma unroll
+      for (int v = 0; v < N; ++v) dq[v] = SUB(P, qR[v], qL[v]);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) qb[v] = MUL(P, 0.5, ADD(P, qL[v], qR[v]));
+      PDE::ncp(2, qb, dq, P, D);
+    }
+  }
+  // A voxel of the column's interior into its slot (plane parity buf).
+  __device__ static void publish(const Smem& S, const DevParams& P, int me, int buf, const double* q, const double* W,
+                                 double lx, double ly) {
+    S.L[me] = lx;
+    S.L[NS + me] = ly;
+    if (HYDRO) {
+      const double ux = PDE::vel(0, q, W), uy = PDE::vel(1, q, W);
+      S.U[me] = ux;
+      S.U[NS + me] = uy;
+      if constexpr (HYDRO) S.X[buf * NT + me] = PDE::press(W);
+      S.X[NXS + buf * NT + me] = cross_term<PDE>(0, q, ux, W, P);
+      S.X[2 * NXS + buf * NT + me] = cross_term<PDE>(1, q, uy, W, P);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) S.Q[v * NS + me] = q[v];
   }
 
   // Ring voxel r of plane z (into ring buffer buf): load, derive, flux and speed
@@ -317,7 +359,7 @@ struct FvTile {
     if (j < TY) { d = 0; y = y0 + j; x = h == 0 ? x0 + TX : x0 - 1; }
     else { d = 1; x = x0 + (j - TY); y = h == 0 ? y0 + TY : y0 - 1; }
     const int64_t e = vox_index(A.patches, A.oct, k, p, x, y, z);
-    double q[NV], W[NW > 0 ? NW : 1], F[N];
+    double q[NV], W[NW > 0 ? NW : 1];
     if (TMA && stb) {
       // the staged strips of this plane: x strips start one voxel before the -x ring voxel
       // and at the +x ring voxel (two wide), y strips hold the ring rows
@@ -333,14 +375,13 @@ struct FvTile {
     const int s = NT + buf * NR + r;
 #pragma unroll
     for (int v = 0; v < NV; ++v) S.Q[v * NS + s] = q[v];
-    double* Fd = d == 0 ? S.Fx : S.Fy;
-    double* Ld = d == 0 ? S.Lx : S.Ly;
-    if (PDE::FLUX) {
-      PDE::flux(d, q, W, A.P, F);
-#pragma unroll
-      for (int v = 0; v < N; ++v) Fd[v * NS + s] = F[v];
+    S.L[d * NS + s] = PDE::speed(d, q, W, A.P);
+    if (HYDRO) {
+      const double u = PDE::vel(d, q, W);
+      S.U[d * NS + s] = u;
+      if constexpr (HYDRO) S.X[2 * NT + buf * NR + r] = PDE::press(W);
+      S.X[(1 + d) * NXS + 2 * NT + buf * NR + r] = cross_term<PDE>(d, q, u, W, A.P);
     }
-    Ld[s] = PDE::speed(d, q, W, A.P);
   }
 
   // maps, bars, abort: TMA staging only (the maps of every level, two mbarriers, the CTA's
@@ -392,50 +433,34 @@ struct FvTile {
     const int fxl = g * FXG + ly * (TX + 1) + lx, fxr = fxl + 1;
     const int fyl = g * FYG + ly * TX + lx, fyu = fyl + TX;
 
-    double Qk[NV];                 // this voxel, current plane
-    double Fzk[N > 0 ? N : 1];     // its z flux (3D)
-    double Lzk = 0.0;              // its z speed
-    double Hzlo[N], Dzlo[N];       // face below the current plane
+    double Qk[NV];            // this voxel, current plane
+    double uzk = 0.0, Lzk = 0.0;  // its z velocity and speed
+    // cell terms along z of the planes below, at and (next iteration) above the current one
+    double pm = 0.0, pk = 0.0, xm = 0.0, xk = 0.0;
+    double Hzlo[N], Dzlo[N];  // face below the current plane
 #pragma unroll
-    for (int v = 0; v < N; ++v) { Hzlo[v] = 0.0; Dzlo[v] = 0.0; Fzk[v] = 0.0; }
+    for (int v = 0; v < N; ++v) { Hzlo[v] = 0.0; Dzlo[v] = 0.0; }
 
     // ---- prologue: plane 0 (and plane -1 for the first z face)
     if (act) {
-      double Wk[NW > 0 ? NW : 1], F[N];
+      double Wk[NW > 0 ? NW : 1];
       load_q<PDE>(A, off + ((int64_t)z0 * p + y) * p + x, Qk);
       derive<PDE, WM>(A, off + ((int64_t)z0 * p + y) * p + x, Qk, Wk);
-      if (DIM == 3 && PDE::FLUX) PDE::flux(2, Qk, Wk, A.P, Fzk);
-      if (PDE::FLUX) {
-        double F2[N];
-        flux_xy<PDE>(Qk, Wk, Fzk, A.P, F, F2);
-#pragma unroll
-        for (int v = 0; v < N; ++v) { S.Fx[v * NS + me] = F[v]; S.Fy[v * NS + me] = F2[v]; }
-      }
-      S.Lx[me] = PDE::speed(0, Qk, Wk, A.P);
-      S.Ly[me] = PDE::speed(1, Qk, Wk, A.P);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) S.Q[v * NS + me] = Qk[v];
+      publish(S, A.P, me, 0, Qk, Wk, PDE::speed(0, Qk, Wk, A.P), PDE::speed(1, Qk, Wk, A.P));
       if (DIM == 3) {
+        uzk = PDE::vel(2, Qk, Wk);
         Lzk = PDE::speed(2, Qk, Wk, A.P);
+        if constexpr (HYDRO) pk = PDE::press(Wk);
+        xk = cross_term<PDE>(2, Qk, uzk, Wk, A.P);
         // plane -1 from the -z neighbour
-        double Qm[NV], Wm[NW > 0 ? NW : 1], Fzm[N];
+        double Qm[NV], Wm[NW > 0 ? NW : 1];
         const int64_t em = vox_index(A.patches, A.oct, k, p, x, y, z0 - 1);
         load_q<PDE>(A, em, Qm);
         derive<PDE, WM>(A, em, Qm, Wm);
-        if (PDE::FLUX) PDE::flux(2, Qm, Wm, A.P, Fzm);
-        const double s = max_nn(PDE::speed(2, Qm, Wm, A.P), Lzk);
-        double dq[N];
-#pragma unroll
-        for (int v = 0; v < N; ++v) {
-          dq[v] = SUB(A.P, Qk[v], Qm[v]);
-          Hzlo[v] = PDE::FLUX ? fma(-s, dq[v], ADD(A.P, Fzm[v], Fzk[v])) : MUL(A.P, -s, dq[v]);
-        }
-        if (PDE::NCP) {
-          double qb[NV];
-#pragma unroll
-          for (int v = 0; v < NV; ++v) qb[v] = MUL(A.P, 0.5, ADD(A.P, Qm[v], Qk[v]));
-          PDE::ncp(2, qb, dq, A.P, Dzlo);
-        }
+        const double um = PDE::vel(2, Qm, Wm);
+        if constexpr (HYDRO) pm = PDE::press(Wm);
+        xm = cross_term<PDE>(2, Qm, um, Wm, A.P);
+        face_z(A.P, Qm, um, PDE::speed(2, Qm, Wm, A.P), Qk, uzk, Lzk, Hzlo, Dzlo);
       }
     }
     if (ring) ring_voxel(A, S, w, tid, p, z0, 0);
@@ -470,27 +495,11 @@ struct FvTile {
           for (int i = 0; i < NW; ++i) prefetch_l2(A.w_in + i * A.vs + e2);
         }
       }
-      // ---- faces of plane kz inside the plane
-      if (act) {
-        face(S, A.P, 0, buf ? xm1 : xm0, me, S.Hx, S.Dx, fxl, FX);
-        face(S, A.P, 1, buf ? ym1 : ym0, me, S.Hy, S.Dy, fyl, FY);
-      }
-      if (tid >= FT0 && tid < FT0 + HALF) {
-        // +x and +y boundary faces of the column: one call with a run-time
-        // direction so that a warp holding both kinds does not diverge
-        const int ft = tid - FT0, gg = ft / RG, j = ft % RG;
-        if (w.patch[gg] >= 0) {
-          const bool isx = j < TY;
-          const int Ls = isx ? gg * TX * TY + j * TX + (TX - 1) : gg * TX * TY + (TY - 1) * TX + (j - TY);
-          const int fidx = isx ? gg * FXG + j * (TX + 1) + TX : gg * FYG + TY * TX + (j - TY);
-          face(S, A.P, isx ? 0 : 1, Ls, NT + buf * NR + ft, isx ? S.Hx : S.Hy, isx ? S.Dx : S.Dy, fidx,
-               isx ? FX : FY);
-        }
-      }
-      // ---- next plane's own voxel (3D): derived quantities, z flux, z face
-      double Qn[NV], Wn[NW > 0 ? NW : 1], Fzn[N], Lzn = 0.0, Lxn = 0.0, Lyn = 0.0, Hzhi[N], Dzhi[N];
+      // ---- loads of the next plane's own voxel (3D)
+      double Qn[NV], Wn[NW > 0 ? NW : 1], uzn = 0.0, Lzn = 0.0, Lxn = 0.0, Lyn = 0.0, pn = 0.0, xn = 0.0;
+      double Hzhi[N], Dzhi[N];
 #pragma unroll
-      for (int v = 0; v < N; ++v) { Hzhi[v] = 0.0; Dzhi[v] = 0.0; Fzn[v] = 0.0; }
+      for (int v = 0; v < N; ++v) { Hzhi[v] = 0.0; Dzhi[v] = 0.0; }
       // TMA: plane zg+1 in buffer kz & 1 (its (kz >> 1)-th use).  A wait that gives up raises
       // the error flag and stops this CTA's later waits (the tile's results are then invalid);
       // the buffer is re-armed only by a thread 0 that saw its phase complete, since a second
@@ -515,30 +524,55 @@ struct FvTile {
         } else {
           load_q<PDE>(A, en, Qn);
         }
-        derive<PDE, WM>(A, en, Qn, Wn);
-        if (PDE::FLUX) PDE::flux(2, Qn, Wn, A.P, Fzn);
-        Lzn = PDE::speed(2, Qn, Wn, A.P);
-        if (speeds_with_z<PDE>()) {
-          Lxn = PDE::speed(0, Qn, Wn, A.P);
-          Lyn = PDE::speed(1, Qn, Wn, A.P);
-        }
-        const double s = max_nn(Lzk, Lzn);
-        double dq[N];
-#pragma unroll
-        for (int v = 0; v < N; ++v) {
-          dq[v] = SUB(A.P, Qn[v], Qk[v]);
-          Hzhi[v] = PDE::FLUX ? fma(-s, dq[v], ADD(A.P, Fzk[v], Fzn[v])) : MUL(A.P, -s, dq[v]);
-        }
-        if (PDE::NCP) {
-          double qb[NV];
-#pragma unroll
-          for (int v = 0; v < NV; ++v) qb[v] = MUL(A.P, 0.5, ADD(A.P, Qk[v], Qn[v]));
-          PDE::ncp(2, qb, dq, A.P, Dzhi);
+        if (WM & 1) derive<PDE, WM>(A, en, Qn, Wn);
+      }
+      // ---- faces of plane kz inside the plane
+      if (act) {
+        face(S, A.P, 0, buf ? xm1 : xm0, me, S.Hx, S.Dx, fxl, FX);
+        face(S, A.P, 1, buf ? ym1 : ym0, me, S.Hy, S.Dy, fyl, FY);
+      }
+      if (tid >= FT0 && tid < FT0 + HALF) {
+        // +x and +y boundary faces of the column: one call with a run-time
+        // direction so that a warp holding both kinds does not diverge
+        const int ft = tid - FT0, gg = ft / RG, j = ft % RG;
+        if (w.patch[gg] >= 0) {
+          const bool isx = j < TY;
+          const int Ls = isx ? gg * TX * TY + j * TX + (TX - 1) : gg * TX * TY + (TY - 1) * TX + (j - TY);
+          const int fidx = isx ? gg * FXG + j * (TX + 1) + TX : gg * FYG + TY * TX + (j - TY);
+          face(S, A.P, isx ? 0 : 1, Ls, NT + buf * NR + ft, isx ? S.Hx : S.Hy, isx ? S.Dx : S.Dy, fidx,
+               isx ? FX : FY);
         }
       }
       // EARLY variant: the ring of plane kz+1 (other ring buffer) overlaps this phase
       if (EARLY && DIM == 3 && kz + 1 < pz && ring) ring_voxel(A, S, w, tid, p, zg + 1, buf ^ 1, S.st[kz & 1]);
+      // ---- what the update of plane kz reads of the earlier stages (loaded before the barrier, which
+      // then hides the loads)
+      const int64_t e = off + ((int64_t)zg * p + y) * p + x;
+      double Rk[N], Pk[N];
+#pragma unroll
+      for (int v = 0; v < N; ++v) { Rk[v] = 0.0; Pk[v] = 0.0; }
+      if (act) {
+#pragma unroll
+        for (int v = 0; v < N; ++v) {
+          if (A.acc && A.form != 1) Rk[v] = A.acc[v * A.vs + e];
+          if (A.q0) Pk[v] = __ldg(A.q0 + v * A.vs + e);
+        }
+      }
       __syncthreads();
+      // ---- z face above the plane (3D): beside the update's integer sums, so that the FP64 pipe
+      // has work in both halves of an iteration
+      if (DIM == 3 && act) {
+        if (!(WM & 1)) derive<PDE, 0>(A, 0, Qn, Wn);
+        uzn = PDE::vel(2, Qn, Wn);
+        Lzn = PDE::speed(2, Qn, Wn, A.P);
+        if constexpr (HYDRO) pn = PDE::press(Wn);
+        xn = cross_term<PDE>(2, Qn, uzn, Wn, A.P);
+        if (speeds_with_z<PDE>()) {
+          Lxn = PDE::speed(0, Qn, Wn, A.P);
+          Lyn = PDE::speed(1, Qn, Wn, A.P);
+        }
+        face_z(A.P, Qk, uzk, Lzk, Qn, uzn, Lzn, Hzhi, Dzhi);
+      }
       // ---- update of plane kz
       if (act) {
         double Sv[N];
@@ -547,49 +581,68 @@ struct FvTile {
           PDE::prims(Qk, A.P, Wk);
           PDE::source(Qk, Wk, A.P, Sv);
         }
-        const int64_t e = off + ((int64_t)zg * p + y) * p + x;
         double res[NV];
-#pragma unroll
-        for (int v = 0; v < N; ++v) {
+        // slots of the x and y neighbours in the cell-term arrays
+        const int cb = buf * NT, rb = 2 * NT + buf * NR + g * RG;
+        const int cxm = lx > 0 ? cb + me - 1 : rb + HALF + ly, cxp = lx < TX - 1 ? cb + me + 1 : rb + ly;
+        const int cym = ly > 0 ? cb + me - TX : rb + HALF + TY + lx, cyp = ly < TY - 1 ? cb + me + TX : rb + TY + lx;
+        for_n<N>([&](auto vc) {
+          constexpr int v = decltype(vc)::value;
           const DevParams& P = A.P;
-          double sum = ADD(P, SUB(P, S.Hx[v * FX + fxr], S.Hx[v * FX + fxl]),
-                           SUB(P, S.Hy[v * FY + fyu], S.Hy[v * FY + fyl]));
-          if (DIM == 3) sum = ADD(P, sum, SUB(P, Hzhi[v], Hzlo[v]));
-          if (PDE::NCP) {
-            double dsum = ADD(P, ADD(P, S.Dx[v * FX + fxr], S.Dx[v * FX + fxl]),
-                              ADD(P, S.Dy[v * FY + fyu], S.Dy[v * FY + fyl]));
-            if (DIM == 3) dsum = ADD(P, dsum, ADD(P, Dzhi[v], Dzlo[v]));
-            sum = ADD(P, sum, dsum);
-          }
           const int64_t ev = v * A.vs + e;
+          // the terms of this quantity's sum over the voxel's faces: the two-sided face values, the
+          // cell terms of the neighbours (those of the voxel itself cancel), the raw sum R of the
+          // earlier stages in the second stage of the stage-sum form
+          constexpr bool MOM = HYDRO && v >= 1 && v <= DIM, EN = HYDRO && v == N - 1;
+          constexpr int NC = DIM + (MOM ? 1 : 0) + (EN ? DIM : 0);
+          constexpr int NPT = NC + (PDE::NCP ? 2 * DIM : 0) + 1;
+          double tp[NPT], tm[NC];
+          tp[0] = S.Hx[v * FX + fxr]; tm[0] = S.Hx[v * FX + fxl];
+          tp[1] = S.Hy[v * FY + fyu]; tm[1] = S.Hy[v * FY + fyl];
+          if constexpr (DIM == 3) { tp[DIM - 1] = Hzhi[v]; tm[DIM - 1] = Hzlo[v]; }
+          if constexpr (MOM) {
+            tp[DIM] = v == 1 ? S.X[cxp] : v == 2 ? S.X[cyp] : pn;
+            tm[DIM] = v == 1 ? S.X[cxm] : v == 2 ? S.X[cym] : pm;
+          }
+          if constexpr (EN) {
+            tp[DIM] = S.X[NXS + cxp]; tm[DIM] = S.X[NXS + cxm];
+            tp[DIM + 1] = S.X[2 * NXS + cyp]; tm[DIM + 1] = S.X[2 * NXS + cym];
+            if constexpr (DIM == 3) { tp[DIM + 2] = xn; tm[DIM + 2] = xm; }
+          }
+          if constexpr (PDE::NCP) {
+            tp[NC] = S.Dx[v * FX + fxr]; tp[NC + 1] = S.Dx[v * FX + fxl];
+            tp[NC + 2] = S.Dy[v * FY + fyu]; tp[NC + 3] = S.Dy[v * FY + fyl];
+            if constexpr (DIM == 3) { tp[NC + 4] = Dzhi[v]; tp[NC + 5] = Dzlo[v]; }
+          }
+          tp[NPT - 1] = !PDE::SRC && A.form == 2 ? Rk[v] : 0.0;
+          const double sum = fx_sum(tp, tm);
           if (!PDE::SRC && A.form != 0) {
             double o;
             if (A.form == 1) {
               o = fma(cS, sum, Qk[v]);
               A.acc[ev] = sum;
             } else if (A.form == 2) {
-              const double t = ADD(P, A.acc[ev], sum);
-              o = fma(cS, t, __ldg(A.q0 + ev));
-              A.acc[ev] = t;
+              o = fma(cS, sum, Pk[v]);
+              A.acc[ev] = sum;
             } else {
-              o = fma(cS, sum, fma(cA, A.acc[ev], __ldg(A.q0 + ev)));
+              o = fma(cS, sum, fma(cA, Rk[v], Pk[v]));
             }
             res[v] = o;
             A.out[ev] = o;
-            continue;
+            return;
           }
           if (A.out) {
             double base = b1 ? Qk[v] : MUL(P, A.b, Qk[v]);
-            if (A.q0) base = fma(A.a, __ldg(A.q0 + ev), base);
+            if (A.q0) base = fma(A.a, Pk[v], base);
             res[v] = PDE::SRC ? fma(gdt, fma(cL, sum, Sv[v]), base) : fma(cS, sum, base);
           }
           if (A.acc) {
-            const double r = PDE::SRC ? fma(ddt, fma(cL, sum, Sv[v]), A.acc[ev]) : fma(cA, sum, A.acc[ev]);
+            const double r = PDE::SRC ? fma(ddt, fma(cL, sum, Sv[v]), Rk[v]) : fma(cA, sum, Rk[v]);
             A.acc[ev] = r;
             if (!A.out) res[v] = r;
           }
           if (A.out) A.out[ev] = res[v];
-        }
+        });
         if (A.lam_out || (WM & 2)) {
 #pragma unroll
           for (int v = N; v < NV; ++v) res[v] = Qk[v];
@@ -609,19 +662,14 @@ struct FvTile {
       // ---- publish plane kz+1 (3D)
       if (DIM == 3 && kz + 1 < pz) {
         if (act) {
-          if (PDE::FLUX) {
-            double F[N], F2[N];
-            flux_xy<PDE>(Qn, Wn, Fzn, A.P, F, F2);
+          publish(S, A.P, me, buf ^ 1, Qn, Wn, speeds_with_z<PDE>() ? Lxn : PDE::speed(0, Qn, Wn, A.P),
+                  speeds_with_z<PDE>() ? Lyn : PDE::speed(1, Qn, Wn, A.P));
 #pragma unroll
-            for (int v = 0; v < N; ++v) { S.Fx[v * NS + me] = F[v]; S.Fy[v * NS + me] = F2[v]; }
-          }
-          S.Lx[me] = speeds_with_z<PDE>() ? Lxn : PDE::speed(0, Qn, Wn, A.P);
-          S.Ly[me] = speeds_with_z<PDE>() ? Lyn : PDE::speed(1, Qn, Wn, A.P);
+          for (int v = 0; v < NV; ++v) Qk[v] = Qn[v];
 #pragma unroll
-          for (int v = 0; v < NV; ++v) { S.Q[v * NS + me] = Qn[v]; Qk[v] = Qn[v]; }
-#pragma unroll
-          for (int v = 0; v < N; ++v) { Fzk[v] = Fzn[v]; Hzlo[v] = Hzhi[v]; Dzlo[v] = Dzhi[v]; }
-          Lzk = Lzn;
+          for (int v = 0; v < N; ++v) { Hzlo[v] = Hzhi[v]; Dzlo[v] = Dzhi[v]; }
+          uzk = uzn; Lzk = Lzn;
+          pm = pk; pk = pn; xm = xk; xk = xn;
         }
         if (!EARLY && ring) ring_voxel(A, S, w, tid, p, zg + 1, buf ^ 1, S.st[kz & 1]);
         __syncthreads();

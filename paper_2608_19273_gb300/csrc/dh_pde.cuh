@@ -99,7 +99,9 @@ __device__ __forceinline__ double max_nn(double a, double b) {
 // dq/dt + div(a q) = 0 with material velocity a (M = 3).  F_d = a_d q, lambda_d = |a_d|.
 struct PdeAdvFlux {
   static constexpr int N = 1, M = 3, NW = 1, DIM = 3;
-  static constexpr bool FLUX = true, NCP = false, SRC = false, SYM = false;
+  static constexpr bool FLUX = true, NCP = false, SRC = false, HYDRO = false;
+  __device__ static constexpr bool moves(int) { return true; }
+  __device__ static double vel(int d, const double* q, const double*) { return sel3(d, q[1], q[2], q[3]); }
   __device__ static void prims(const double*, const DevParams&, double*) {}
   __device__ static void flux(int d, const double* q, const double*, const DevParams& P, double* F) {
     F[0] = MUL(P, sel3(d, q[1], q[2], q[3]), q[0]);
@@ -114,7 +116,9 @@ struct PdeAdvFlux {
 // dq/dt + a . grad q = 0 (non-conservative form, F = 0): B_d = a_d.
 struct PdeAdvNcp {
   static constexpr int N = 1, M = 3, NW = 1, DIM = 3;
-  static constexpr bool FLUX = false, NCP = true, SRC = false, SYM = false;
+  static constexpr bool FLUX = false, NCP = true, SRC = false, HYDRO = false;
+  __device__ static constexpr bool moves(int) { return false; }
+  __device__ static double vel(int d, const double* q, const double*) { return sel3(d, q[1], q[2], q[3]); }
   __device__ static constexpr bool needs_grad(int, int v) { return v == 0; }
   __device__ static void prims(const double*, const DevParams&, double*) {}
   __device__ static void flux(int, const double*, const double*, const DevParams&, double*) {}
@@ -130,11 +134,19 @@ struct PdeAdvNcp {
 
 // ---------------------------------------------------------------- Euler
 // Ideal-gas Euler equations in DIM dimensions: Q = (rho, rho u_k, E).
-// W = (u_0 .. u_{DIM-1}, p, c, H = E + p): one reciprocal and one square root per voxel.
+// W = (u_0 .. u_{DIM-1}, p, c): one reciprocal and one square root per voxel.
 template <int D_>
 struct PdeEuler {
-  static constexpr int DIM = D_, N = D_ + 2, M = 0, NW = D_ + 3;
-  static constexpr bool FLUX = true, NCP = false, SRC = false, SYM = true;
+  static constexpr int DIM = D_, N = D_ + 2, M = 0, NW = D_ + 2;
+  static constexpr bool FLUX = true, NCP = false, SRC = false, HYDRO = true;
+  // F_d = Q u_d + p e_d + (p u_d) e_E: every quantity moves with u_d; the pressure terms are the
+  // cell values press and cross.
+  __device__ static constexpr bool moves(int) { return true; }
+  __device__ static double vel(int d, const double*, const double* w) {
+    return (DIM == 3) ? sel3(d, w[0], w[1], w[DIM == 3 ? 2 : 0]) : (d == 0 ? w[0] : w[1]);
+  }
+  __device__ static double press(const double* w) { return w[DIM]; }
+  __device__ static double cross(const double*, double u, const double* w, const DevParams& P) { return MUL(P, w[DIM], u); }
   __device__ static void prims(const double* q, const DevParams& P, double* w) {
     const double r = recip_nr(q[0]);
     w[0] = MUL(P, q[1], r);
@@ -147,41 +159,15 @@ struct PdeEuler {
     const double p = MUL(P, P.gm1, fma(-0.5, kin, q[DIM + 1]));
     w[DIM] = p;
     w[DIM + 1] = sqrt_pos(MUL(P, MUL(P, P.gamma, p), r));
-    w[DIM + 2] = ADD(P, q[DIM + 1], p);
   }
-  // The momentum flux rho u_k u_d is symmetric in (k, d); every direction forms
-  // it as m_min(k,d) u_max(k,d), so the x, y and z fluxes of one voxel share
-  // their off-diagonal products bit for bit (flux_xy).
   __device__ static void flux(int d, const double* q, const double* w, const DevParams& P, double* F) {
-    const double u = (DIM == 3) ? sel3(d, w[0], w[1], w[DIM == 3 ? 2 : 0]) : (d == 0 ? w[0] : w[1]);
-    const double p = w[DIM];
-    F[0] = (DIM == 3) ? sel3(d, q[1], q[2], q[DIM == 3 ? 3 : 1]) : (d == 0 ? q[1] : q[2]);
+    const double u = vel(d, q, w), p = w[DIM];
 #pragma unroll
-    for (int k = 0; k < DIM; ++k)
-      F[1 + k] = fma(k < d ? q[1 + k] : F[0], k < d ? u : w[k], d == k ? p : P.zero);
-    F[DIM + 1] = MUL(P, w[DIM + 2], u);
-  }
-  // F_x and F_y of a voxel whose F_z (3D) is already formed: the same values as
-  // flux(0) and flux(1), with the products m_x u_y, m_x u_z, m_y u_z formed once.
-  __device__ static void flux_xy(const double* q, const double* w, const double* Fz, const DevParams& P, double* Fx,
-                                 double* Fy) {
-    const double p = w[DIM], cxy = MUL(P, q[1], w[1]);
-    Fx[0] = q[1];
-    Fx[1] = fma(q[1], w[0], p);
-    Fx[2] = cxy;
-    Fy[0] = q[2];
-    Fy[1] = cxy;
-    Fy[2] = fma(q[2], w[1], p);
-    if (DIM == 3) {
-      Fx[DIM == 3 ? 3 : 0] = Fz[1];
-      Fy[DIM == 3 ? 3 : 0] = Fz[2];
-    }
-    Fx[DIM + 1] = MUL(P, w[DIM + 2], w[0]);
-    Fy[DIM + 1] = MUL(P, w[DIM + 2], w[1]);
+    for (int v = 0; v < N; ++v) F[v] = v == 1 + d ? fma(q[v], u, p) : MUL(P, q[v], u);
+    F[N - 1] = MUL(P, ADD(P, q[N - 1], p), u);
   }
   __device__ static double speed(int d, const double*, const double* w, const DevParams& P) {
-    const double u = (DIM == 3) ? sel3(d, w[0], w[1], w[DIM == 3 ? 2 : 0]) : (d == 0 ? w[0] : w[1]);
-    return ADD(P, fabs(u), w[DIM + 1]);
+    return ADD(P, fabs(vel(d, nullptr, w)), w[DIM + 1]);
   }
   __device__ static void ncp(int, const double*, const double*, const DevParams&, double*) {}
   __device__ static void source(const double*, const double*, const DevParams&, double*) {}
@@ -201,7 +187,12 @@ using PdeEuler3 = PdeEuler<3>;
 // (cs is folded under the square root: one square root per direction, none per voxel).
 struct PdeSRHD {
   static constexpr int N = 5, M = 5, NW = 8, DIM = 3;
-  static constexpr bool FLUX = true, NCP = false, SRC = false, SYM = true;
+  static constexpr bool FLUX = true, NCP = false, SRC = false, HYDRO = true;
+  // D and S move with v_d; the flux S_d - D v_d of tau is a cell value (cross), and so is p.
+  __device__ static constexpr bool moves(int v) { return v < 4; }
+  __device__ static double vel(int d, const double*, const double* w) { return sel3(d, w[0], w[1], w[2]); }
+  __device__ static double press(const double* w) { return w[3]; }
+  __device__ static double cross(double D, double Sd, double v) { return fma(-D, v, Sd); }
   __device__ static void prims(const double* q, const DevParams& P, double* w) {
     const double rho = q[5], vx = q[6], vy = q[7], vz = q[8], p = q[9];
     const double v2 = fma(vx, vx, fma(vy, vy, MUL(P, vz, vz)));
@@ -214,28 +205,12 @@ struct PdeSRHD {
     w[6] = c0;
     w[7] = recip_nr(c0);
   }
-  // S_k v_d = rho h W^2 v_k v_d is symmetric in (k, d); every direction forms
-  // it as S_min(k,d) v_max(k,d) (shared products, flux_xy).
   __device__ static void flux(int d, const double* q, const double* w, const DevParams& P, double* F) {
     const double v = sel3(d, w[0], w[1], w[2]), p = w[3], Sd = sel3(d, q[1], q[2], q[3]);
     F[0] = MUL(P, q[0], v);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) F[1 + k] = fma(k < d ? q[1 + k] : Sd, k < d ? v : w[k], d == k ? p : P.zero);
-    F[4] = fma(-q[0], v, Sd);
-  }
-  __device__ static void flux_xy(const double* q, const double* w, const double* Fz, const DevParams& P, double* Fx,
-                                 double* Fy) {
-    const double p = w[3], cxy = MUL(P, q[1], w[1]);
-    Fx[0] = MUL(P, q[0], w[0]);
-    Fx[1] = fma(q[1], w[0], p);
-    Fx[2] = cxy;
-    Fx[3] = Fz[1];
-    Fx[4] = fma(-q[0], w[0], q[1]);
-    Fy[0] = MUL(P, q[0], w[1]);
-    Fy[1] = cxy;
-    Fy[2] = fma(q[2], w[1], p);
-    Fy[3] = Fz[2];
-    Fy[4] = fma(-q[0], w[1], q[2]);
+    for (int k = 0; k < 3; ++k) F[1 + k] = k == d ? fma(q[1 + k], v, p) : MUL(P, q[1 + k], v);
+    F[4] = cross(q[0], Sd, v);
   }
   __device__ static double speed(int d, const double*, const double* w, const DevParams& P) {
     const double v = sel3(d, w[0], w[1], w[2]), omc = w[4];
@@ -266,7 +241,7 @@ struct PdeSRHD {
 // S = (Pi, -gamma Pi, 0, 0, 0).  Material: c (M = 1).  lambda_d = c.
 struct PdeWave {
   static constexpr int N = 5, M = 1, NW = 1, DIM = 3;
-  static constexpr bool FLUX = false, NCP = true, SRC = true, SYM = false;
+  static constexpr bool FLUX = false, NCP = true, SRC = true;
   __device__ static constexpr bool needs_grad(int d, int v) { return v == 1 || v == 2 + d; }
   __device__ static void prims(const double*, const DevParams&, double*) {}
   __device__ static void flux(int, const double*, const double*, const DevParams&, double*) {}
@@ -298,12 +273,36 @@ struct PdeWave {
 // alpha at 55, beta at 56..58.  lambda_d = alpha + |beta^d|.
 struct PdeGW59 {
   static constexpr int N = 59, M = 0, NW = 1, DIM = 3;
-  static constexpr bool FLUX = false, NCP = true, SRC = true, SYM = false;
+  static constexpr bool FLUX = false, NCP = true, SRC = true;
   __device__ static void prims(const double*, const DevParams&, double*) {}
   __device__ static double speed(int d, const double* q, const double*, const DevParams&) {
     return q[55] + fabs(sel3(d, q[56], q[57], q[58]));
   }
 };
+
+// The cell value that a system adds to the face differences of its last quantity (the flux of the
+// energy beyond its transport): p u_d for Euler, S_d - D v_d for SRHD (q: N quantities, u = vel).
+template <class PDE>
+__device__ __forceinline__ double cross_term(int d, const double* q, double u, const double* w, const DevParams& P) {
+  if constexpr (std::is_same<PDE, PdeSRHD>::value) return PdeSRHD::cross(q[0], sel3(d, q[1], q[2], q[3]), u);
+  else if constexpr (PDE::HYDRO) return PDE::cross(q, u, w, P);
+  else return 0.0;
+}
+
+// The part of twice the Rusanov flux that needs both sides of a face,
+//   F_L + F_R - s (Q_R - Q_L) = Q_L (u_L + s) + Q_R (u_R - s) + cell terms,  s = max(lambda_L, lambda_R):
+// two operations per quantity that moves with the velocity u (and s (Q_L - Q_R) for the others).
+// The cell terms (pressure, cross_term) enter the sums over a voxel's faces directly (face_sum),
+// where those of the voxel itself cancel.
+template <class PDE>
+__device__ __forceinline__ void rusanov(const DevParams& P, const double* qL, double uL, double lL, const double* qR,
+                                        double uR, double lR, double* H) {
+  const double s = max_nn(lL, lR);
+  const double a = ADD(P, uL, s), b = SUB(P, uR, s);
+#pragma unroll
+  for (int v = 0; v < PDE::N; ++v)
+    H[v] = PDE::moves(v) ? fma(qR[v], b, MUL(P, qL[v], a)) : MUL(P, s, SUB(P, qL[v], qR[v]));
+}
 
 // The largest characteristic speed of a voxel over its dim directions (SRHD: the speed of the
 // direction of the largest |v_d|, which is the largest).

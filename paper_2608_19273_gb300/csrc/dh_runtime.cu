@@ -241,7 +241,7 @@ static bool w_reuse(dh_plan* plan, int scheme, int rk, int n_steps, double cfl) 
 
 // The plan's two W arenas (allocated once, on first use, and kept by the plan).
 static dh_status w_chain(dh_plan* plan, int n_steps, WChain& wc) {
-  const size_t nw = (size_t)(plan->dim + 3) * (size_t)plan->var_stride;
+  const size_t nw = (size_t)(plan->dim + 2) * (size_t)plan->var_stride;
   if (!plan->d_w) DH_TRY(cuda_error(cudaMalloc(&plan->d_w, 2 * sizeof(double) * nw), "W arenas"));
   wc.on = true;
   wc.next = 0;
