@@ -9,23 +9,25 @@
 // upper ends).  One voxel per thread.  Every item keeps within the limits below (checked on the
 // host when the plan is made).
 //   1. Every cell of the box and its one-voxel face halo (edges and corners are never read) is
-//      loaded into shared memory with its derived quantities W (read from the W arena of the
-//      stage input, or computed).
-//   2. Per direction d: every line cell of d (the box and its halo layers at both ends along d) forms
-//      its flux F_d and speed lambda_d into the line arrays; after a barrier every face along d
-//      is formed once (one per thread) into the face arrays; after another barrier every voxel
-//      adds the difference of its two faces.
-//   3. The stage combination, W of the result and lambda of the result as in the marching stage.
-// Shared memory: box cells x (N + M quantities, W), line cells x (F_d, lambda_d), faces x (the
-// face values, and the non-conservative products of NCP systems); 70.7 KB for the Euler
-// equations in 3D, three CTAs per SM.
+//      loaded into shared memory with its velocity, pressure and sound speed (from the W arena of
+//      the stage input, or computed; SRHD: the speeds of the directions it is used in).
+//   2. After a barrier every face of all directions is formed once, one per thread and direction
+//      (rusanov, the two-sided part of twice the flux), into the face arrays.
+//   3. After another barrier every voxel sums its faces and its neighbours' cell terms in fixed
+//      point (fx_sum); the stage combination, W of the result and lambda of the result as in the
+//      marching stage.
+// Shared memory: box cells x (N quantities, velocity, pressure, sound speed or speeds), faces x N
+// and direction; 71.7 KB for the Euler equations in 3D, three CTAs per SM.
+// Bound by the FP64 pipe: about 81 instructions a voxel, 144 when every line cell's flux was formed (the
+// face halo of a 6^3 box is as many cells as the box), direction after direction with two barriers
+// each, and every face sum was FP64.  16,384 patches of 6^3, two SSP-RK3 steps: 6.71 -> 4.97 ms (the FP64
+// instructions alone: 3.4); 4096 of 3^3: 0.23 ms.
 #pragma once
 
 namespace dh {
 
 constexpr int ANY_NT = 256;      // threads per CTA; voxels per item at most
 constexpr int ANY_SLOTS = 512;   // box cells with halo (all groups) per item
-constexpr int ANY_LINES = 320;   // line cells of one direction per item
 constexpr int ANY_FACES = 256;   // faces of one direction per item (one per thread)
 
 // Integer division by a run-time divisor without the integer divide sequence: for
@@ -42,18 +44,26 @@ struct ADiv {
 template <class PDE>
 struct FvAny {
   static constexpr int N = PDE::N, NV = PDE::N + PDE::M, NW = PDE::NW > 0 ? PDE::NW : 1, DIM = PDE::DIM;
+  static constexpr bool HYDRO = PDE::HYDRO;
+  // speeds: SRHD keeps the three of a cell (a square root each), Euler its sound speed (one addition
+  // per use; with three arrays more only two CTAs fit), advection has them from the velocity
+  static constexpr bool SRHD = std::is_same<PDE, PdeSRHD>::value;
+  static constexpr int NL = SRHD ? 3 : (HYDRO ? 1 : 0);
+  static constexpr int NC = N + DIM + (HYDRO ? 1 : 0) + NL;  // values kept per cell
   static constexpr int NF = PDE::NCP ? 2 : 1;  // face arrays: flux (and non-conservative product)
   static constexpr size_t SMEM =
-      sizeof(double) * ((size_t)ANY_SLOTS * (NV + NW) + (size_t)ANY_LINES * (N + 1) + (size_t)ANY_FACES * NF * N);
+      sizeof(double) * ((size_t)ANY_SLOTS * NC + (size_t)ANY_FACES * NF * N * DIM);
+  static constexpr int CTAS = SMEM <= 74 * 1024 ? 3 : 2;
 
   template <int WM>
   __device__ static void run(const FvArgs& A, const AnyWork& w, double* smem, double& lam_thread) {
-    double* Q = smem;                 // [NV][ANY_SLOTS]: box cells
-    double* Wc = Q + NV * ANY_SLOTS;  // [NW][ANY_SLOTS]
-    double* F = Wc + NW * ANY_SLOTS;  // [N][ANY_LINES]: line cells of one direction
-    double* L = F + N * ANY_LINES;    // [ANY_LINES]
-    double* H = L + ANY_LINES;        // [N][ANY_FACES]: face values of one direction
-    double* Dn = H + N * ANY_FACES;   // [N][ANY_FACES]: non-conservative products (NCP systems)
+    double* Q = smem;                      // [N][ANY_SLOTS]: box cells
+    double* U = Q + N * ANY_SLOTS;         // [DIM][ANY_SLOTS]: velocity (advection: the material)
+    double* Pr = U + DIM * ANY_SLOTS;      // [ANY_SLOTS]: pressure (HYDRO)
+    double* L = Pr + (HYDRO ? ANY_SLOTS : 0);  // [NL][ANY_SLOTS]
+    double* H = L + NL * ANY_SLOTS;        // [DIM][N][ANY_FACES]: face values
+    double* Dn = H + DIM * N * ANY_FACES;  // [DIM][N][ANY_FACES]: non-conservative products (NCP systems)
+    __shared__ double sc[3];               // the item's -1/(2 dx) (faces hold twice the flux), g dt and d dt times it
     const DevParams& P = A.P;
     const int bx = w.bx, by = w.by, bz = DIM == 3 ? w.bz : 1, ng = w.ng;
     const int SX = bx + 2, SY = by + 2, SZ = DIM == 3 ? bz + 2 : 1;
@@ -64,8 +74,12 @@ struct FvAny {
     const bool act = g < ng;
     const int lx = li % bx, ly = (li / bx) % by, lz = li / (bx * by);
     const int p = A.patches[w.patch[0]].p;  // every group or block member of an item has the same p
-    const double dt = *A.dt_dev;             // read before the lambda epilogue may rewrite it
-    const double gdt = A.g * dt, ddt = A.d * dt;
+    if (tid == 0) {
+      const double dt = *A.dt_dev;  // read before the lambda epilogue may rewrite it
+      sc[0] = -0.5 / A.patches[w.patch[0]].dx;  // (every patch of an item has the same dx)
+      sc[1] = A.g * dt * sc[0];
+      sc[2] = A.d * dt * sc[0];
+    }
 
     // 1. the box and its face halo, with W: the cells that are read, enumerated group by group as
     //    the box (x fastest), then the two halo layers across x, y and z (edges and corners are
@@ -75,7 +89,7 @@ struct FvAny {
     const ADiv dCG(CG), dBX(bx), dBXY(bx * by), dBY(by), dHX(HX), dHY(HY), dHZ(HZ > 0 ? HZ : 1);
     for (int j = tid; j < ng * CG; j += ANY_NT) {
       const int gg = dCG.q(j);
-      int r = j - gg * CG, cx, cy, cz;
+      int r = j - gg * CG, cx, cy, cz, hd = -1;  // hd: the halo cell's direction
       if (r < nvg) {
         cz = DIM == 3 ? dBXY.q(r) : 0;
         const int rxy = r - cz * bx * by;
@@ -83,17 +97,20 @@ struct FvAny {
         cx = rxy - cy * bx;
       } else if ((r -= nvg) < 2 * HX) {
         const int side = dHX.q(r), t = r - side * HX;
+        hd = 0;
         cx = side ? bx : -1;
         cz = dBY.q(t);
         cy = t - cz * by;
       } else if ((r -= 2 * HX) < 2 * HY) {
         const int side = dHY.q(r), t = r - side * HY;
+        hd = 1;
         cy = side ? by : -1;
         cz = dBX.q(t);
         cx = t - cz * bx;
       } else {
         r -= 2 * HY;
         const int side = dHZ.q(r), t = r - side * HZ;
+        hd = 2;
         cz = side ? bz : -1;
         cy = dBX.q(t);
         cx = t - cy * bx;
@@ -121,90 +138,57 @@ struct FvAny {
         PDE::prims(q, P, W);
       }
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Q[v * ANY_SLOTS + s] = q[v];
+      for (int v = 0; v < N; ++v) Q[v * ANY_SLOTS + s] = q[v];
 #pragma unroll
-      for (int i = 0; i < NW; ++i) Wc[i * ANY_SLOTS + s] = W[i];
+      for (int d = 0; d < DIM; ++d) U[d * ANY_SLOTS + s] = PDE::vel(d, q, W);
+      if constexpr (HYDRO) Pr[s] = PDE::press(W);
+      if constexpr (SRHD) {
+#pragma unroll
+        for (int d = 0; d < DIM; ++d)
+          if (hd < 0 || hd == d) L[d * ANY_SLOTS + s] = PDE::speed(d, q, W, P);
+      } else if constexpr (HYDRO) {
+        L[s] = W[DIM + 1];
+      }
     }
     __syncthreads();
 
-    // 2. per direction: line fluxes and speeds, then this voxel's two faces
-    const int me = g * SG + ((DIM == 3 ? lz + 1 : 0) * SY + (ly + 1)) * SX + (lx + 1);
-    double sum[N], dsum[N];
+    // 2. every face once, one per thread and direction, in x-fastest order (consecutive threads touch
+    //    consecutive cells: no shared-memory bank conflicts in any direction).  The face grid of a
+    //    direction is the voxel grid with one more layer along it: the face at c_d = pos lies
+    //    between the cells at pos - 1 and pos (pos = 0 and pos = b_d take a halo cell).
+    const int cst[3] = {1, SX, SX * SY};  // box cells along x, y, z
 #pragma unroll
-    for (int v = 0; v < N; ++v) { sum[v] = 0.0; dsum[v] = 0.0; }
-#pragma unroll 1
     for (int d = 0; d < DIM; ++d) {
-      // the line cells of d (the box and the halo layer at each of its ends along d) of every
-      // group, x fastest; their fluxes and speeds go to the line arrays at index j
-      const int LX = bx + 2 * (d == 0), LY = by + 2 * (d == 1), LZ = DIM == 3 ? bz + 2 * (d == 2) : 1;
-      const int LG = LX * LY * LZ;
-      const ADiv dLG(LG), dLX(LX), dLY(LY);
-      for (int j = tid; j < ng * LG; j += ANY_NT) {
-        const int gg = dLG.q(j), r = j - gg * LG, t = dLX.q(r), hi = dLY.q(t);
-        const int cx = r - t * LX - (d == 0), cy = t - hi * LY - (d == 1), cz = hi - (d == 2);
-        const int s = gg * SG + ((DIM == 3 ? cz + 1 : 0) * SY + (cy + 1)) * SX + (cx + 1);
-        double q[NV], W[NW], Fd[N];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) q[v] = Q[v * ANY_SLOTS + s];
-#pragma unroll
-        for (int i = 0; i < NW; ++i) W[i] = Wc[i * ANY_SLOTS + s];
-        if (PDE::FLUX) {
-          PDE::flux(d, q, W, P, Fd);
-#pragma unroll
-          for (int v = 0; v < N; ++v) F[v * ANY_LINES + j] = Fd[v];
-        }
-        L[j] = PDE::speed(d, q, W, P);
-      }
-      __syncthreads();
-      // every face along d once, one per thread, in x-fastest order (consecutive threads touch
-      // consecutive cells: no shared-memory bank conflicts in any direction).  The face grid is
-      // the voxel grid with one more layer along d: the face at c_d = pos lies between the cells
-      // at pos - 1 and pos (pos = 0 and pos = b_d take a halo cell).
       const int FX = bx + (d == 0), FY = by + (d == 1), FZ = DIM == 3 ? bz + (d == 2) : 1;
       const int FG = FX * FY * FZ;  // faces per group
-      {
-        const int st = d == 0 ? 1 : (d == 1 ? SX : SX * SY), lst = d == 0 ? 1 : (d == 1 ? LX : LX * LY);
+      if (tid < ng * FG) {
         const ADiv dFG(FG), dFX(FX), dFY(FY);
-        const int fi = tid;
-        if (fi < ng * FG) {
-          const int gg = dFG.q(fi), r = fi - gg * FG, t = dFX.q(r), cz = dFY.q(t);
-          const int cx = r - t * FX, cy = t - cz * FY;
-          const int cR = gg * SG + ((DIM == 3 ? cz + 1 : 0) * SY + (cy + 1)) * SX + (cx + 1), cLf = cR - st;
-          // the same two cells in the line arrays (line coordinates are shifted by one along d)
-          const int jR = gg * LG + ((DIM == 3 ? cz + (d == 2) : 0) * LY + (cy + (d == 1))) * LX + (cx + (d == 0));
-          const int jL = jR - lst;
-          const double sf = max_nn(L[jL], L[jR]);
-          double dq[N];
+        const int gg = dFG.q(tid), r = tid - gg * FG, t = dFX.q(r), cz = dFY.q(t);
+        const int cx = r - t * FX, cy = t - cz * FY;
+        const int cR = gg * SG + ((DIM == 3 ? cz + 1 : 0) * SY + (cy + 1)) * SX + (cx + 1), cLf = cR - cst[d];
+        double qL[N], qR[N], h[N];
 #pragma unroll
-          for (int v = 0; v < N; ++v) {
-            dq[v] = SUB(P, Q[v * ANY_SLOTS + cR], Q[v * ANY_SLOTS + cLf]);
-            H[v * ANY_FACES + fi] = PDE::FLUX ? fma(-sf, dq[v], ADD(P, F[v * ANY_LINES + jL], F[v * ANY_LINES + jR]))
-                                              : MUL(P, -sf, dq[v]);
-          }
-          if (PDE::NCP) {
-            double qb[NV], Dv[N];
+        for (int v = 0; v < N; ++v) { qL[v] = Q[v * ANY_SLOTS + cLf]; qR[v] = Q[v * ANY_SLOTS + cR]; }
+        const double uL = U[d * ANY_SLOTS + cLf], uR = U[d * ANY_SLOTS + cR];
+        double lL = fabs(uL), lR = fabs(uR);
+        if constexpr (SRHD) { lL = L[d * ANY_SLOTS + cLf]; lR = L[d * ANY_SLOTS + cR]; }
+        else if constexpr (HYDRO) { lL = ADD(P, lL, L[cLf]); lR = ADD(P, lR, L[cR]); }
+        rusanov<PDE>(P, qL, uL, lL, qR, uR, lR, h);
 #pragma unroll
-            for (int v = 0; v < NV; ++v) qb[v] = MUL(P, 0.5, ADD(P, Q[v * ANY_SLOTS + cLf], Q[v * ANY_SLOTS + cR]));
-            PDE::ncp(d, qb, dq, P, Dv);
+        for (int v = 0; v < N; ++v) H[(d * N + v) * ANY_FACES + tid] = h[v];
+        if constexpr (PDE::NCP) {
+          double qb[NV], dq[N], Dv[N];
 #pragma unroll
-            for (int v = 0; v < N; ++v) Dn[v * ANY_FACES + fi] = Dv[v];
-          }
+          for (int v = 0; v < N; ++v) { dq[v] = SUB(P, qR[v], qL[v]); qb[v] = MUL(P, 0.5, ADD(P, qL[v], qR[v])); }
+#pragma unroll
+          for (int v = 0; v < PDE::M; ++v) qb[N + v] = MUL(P, 0.5, ADD(P, U[v * ANY_SLOTS + cLf], U[v * ANY_SLOTS + cR]));
+          PDE::ncp(d, qb, dq, P, Dv);
+#pragma unroll
+          for (int v = 0; v < N; ++v) Dn[(d * N + v) * ANY_FACES + tid] = Dv[v];
         }
       }
-      __syncthreads();
-      if (act) {
-        // this voxel's two faces along d: face coordinates pos = l_d and l_d + 1
-        const int fm = g * FG + ((DIM == 3 ? lz : 0) * FY + ly) * FX + lx;
-        const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
-#pragma unroll
-        for (int v = 0; v < N; ++v) {
-          sum[v] = ADD(P, sum[v], SUB(P, H[v * ANY_FACES + fp], H[v * ANY_FACES + fm]));
-          if (PDE::NCP) dsum[v] = ADD(P, dsum[v], ADD(P, Dn[v * ANY_FACES + fp], Dn[v * ANY_FACES + fm]));
-        }
-      }
-      // (the next direction writes F and L first, which no thread reads any more, then -- after a
-      // barrier -- H)
     }
+    __syncthreads();
 
     // 3. stage combination, W and lambda of the result
     if (!act) return;
@@ -217,51 +201,79 @@ struct FvAny {
       k = __ldg(w.patch + g);
       x = w.x0 + lx; y = w.y0 + ly; z = DIM == 3 ? w.z0 + lz : 0;
     }
-    const double cL = -0.5 / A.patches[k].dx;  // faces hold twice the flux
-    const double cS = gdt * cL, cA = ddt * cL;
+    const double cS = sc[1], cA = sc[2];
     const bool b1 = A.b == 1.0;
     const int pk = w.mp > 0 ? w.mp : p;
     const int64_t e = A.patches[k].offset + ((int64_t)z * pk + y) * pk + x;
-    double Qk[NV], Sv[N], res[NV];
+    const int me = g * SG + ((DIM == 3 ? lz + 1 : 0) * SY + (ly + 1)) * SX + (lx + 1);
+    double Qk[NV], res[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) Qk[v] = Q[v * ANY_SLOTS + me];
-    if (PDE::SRC) {
-      double Wk[NW];
-      PDE::prims(Qk, P, Wk);
-      PDE::source(Qk, Wk, P, Sv);
+    for (int v = 0; v < N; ++v) Qk[v] = Q[v * ANY_SLOTS + me];
+#pragma unroll
+    for (int v = 0; v < PDE::M; ++v) Qk[N + v] = HYDRO ? __ldg(A.mat + v * A.vs + e) : U[v * ANY_SLOTS + me];
+    static_assert(!PDE::SRC, "systems without a source term");
+    // this voxel's faces in the face arrays: below along x, y, z, and the steps to those above
+    int fm[DIM], fs[DIM];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+      const int FX = bx + (d == 0), FY = by + (d == 1), FZ = DIM == 3 ? bz + (d == 2) : 1;
+      fm[d] = g * FX * FY * FZ + ((DIM == 3 ? lz : 0) * FY + ly) * FX + lx;
+      fs[d] = d == 0 ? 1 : (d == 1 ? FX : FX * FY);
     }
-#pragma unroll
-    for (int v = 0; v < N; ++v) {
-      const double s = PDE::NCP ? ADD(P, sum[v], dsum[v]) : sum[v];
+    for_n<N>([&](auto vc) {
+      constexpr int v = decltype(vc)::value;
+      // the terms as in the marching stage: faces, cell terms of the neighbours, the raw sum R
+      constexpr bool MOM = HYDRO && v >= 1 && v <= DIM, EN = HYDRO && v == N - 1;
+      constexpr int NT = DIM + (MOM ? 1 : 0) + (EN ? DIM : 0);
+      constexpr int NPT = NT + (PDE::NCP ? 2 * DIM : 0) + 1;
       const int64_t ev = v * A.vs + e;
-      if (!PDE::SRC && A.form != 0) {
-        double o;
-        if (A.form == 1) {
-          o = fma(cS, s, Qk[v]);
-          A.acc[ev] = s;
-        } else if (A.form == 2) {
-          const double t = ADD(P, A.acc[ev], s);
-          o = fma(cS, t, __ldg(A.q0 + ev));
-          A.acc[ev] = t;
-        } else {
-          o = fma(cS, s, fma(cA, A.acc[ev], __ldg(A.q0 + ev)));
+      double tp[NPT], tm[NT];
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) {
+        const double* Hv = H + (d * N + v) * ANY_FACES + fm[d];
+        tp[d] = Hv[fs[d]]; tm[d] = Hv[0];
+        if constexpr (PDE::NCP) {
+          const double* Dv = Dn + (d * N + v) * ANY_FACES + fm[d];
+          tp[NT + 2 * d] = Dv[fs[d]]; tp[NT + 2 * d + 1] = Dv[0];
         }
+        if constexpr (EN) {
+          const int cp = me + cst[d], cm = me - cst[d];
+          const double up = U[d * ANY_SLOTS + cp], um = U[d * ANY_SLOTS + cm];
+          if constexpr (SRHD) {
+            tp[DIM + d] = PdeSRHD::cross(Q[cp], Q[(1 + d) * ANY_SLOTS + cp], up);
+            tm[DIM + d] = PdeSRHD::cross(Q[cm], Q[(1 + d) * ANY_SLOTS + cm], um);
+          } else {
+            tp[DIM + d] = MUL(P, Pr[cp], up);
+            tm[DIM + d] = MUL(P, Pr[cm], um);
+          }
+        }
+      }
+      if constexpr (MOM) { tp[DIM] = Pr[me + cst[v - 1]]; tm[DIM] = Pr[me - cst[v - 1]]; }
+      const double R = A.acc && A.form != 1 ? A.acc[ev] : 0.0;
+      tp[NPT - 1] = A.form == 2 ? R : 0.0;
+      const double s = fx_sum(tp, tm);
+      if (A.form != 0) {
+        double o;
+        if (A.form == 1) o = fma(cS, s, Qk[v]);
+        else if (A.form == 2) o = fma(cS, s, __ldg(A.q0 + ev));
+        else o = fma(cS, s, fma(cA, R, __ldg(A.q0 + ev)));
+        if (A.form != 3) A.acc[ev] = s;
         res[v] = o;
         A.out[ev] = o;
-        continue;
+        return;
       }
       if (A.out) {
         double base = b1 ? Qk[v] : MUL(P, A.b, Qk[v]);
         if (A.q0) base = fma(A.a, __ldg(A.q0 + ev), base);
-        res[v] = PDE::SRC ? fma(gdt, fma(cL, s, Sv[v]), base) : fma(cS, s, base);
+        res[v] = fma(cS, s, base);
       }
       if (A.acc) {
-        const double r = PDE::SRC ? fma(ddt, fma(cL, s, Sv[v]), A.acc[ev]) : fma(cA, s, A.acc[ev]);
+        const double r = fma(cA, s, R);
         A.acc[ev] = r;
         if (!A.out) res[v] = r;
       }
       if (A.out) A.out[ev] = res[v];
-    }
+    });
     if (A.lam_out || (WM & 2)) {
 #pragma unroll
       for (int v = N; v < NV; ++v) res[v] = Qk[v];
@@ -281,10 +293,11 @@ struct FvAny {
 };
 
 template <class PDE, int WM>
-__global__ void __launch_bounds__(ANY_NT) k_fv_any(const __grid_constant__ FvArgs A, const AnyWork* __restrict__ work) {
+__global__ void __launch_bounds__(ANY_NT, FvAny<PDE>::CTAS) k_fv_any(const __grid_constant__ FvArgs A, const AnyWork* __restrict__ work) {
   extern __shared__ __align__(128) double smem[];
   double lam = 0.0;
-  FvAny<PDE>::template run<WM>(A, work[blockIdx.x], smem, lam);
+  const FvArgs R = with_reg_params(A);
+  FvAny<PDE>::template run<WM>(R, work[blockIdx.x], smem, lam);
   if (A.lam_out) publish_lambda(lam, A.lam_out, A.red, A.dt_next, A.cfl, A.dx_dim);
 }
 
