@@ -50,7 +50,6 @@
 #include <algorithm>
 #include <type_traits>
 
-#include <utility>
 
 #include "dh_fixed.cuh"
 #include "dh_internal.cuh"
@@ -89,26 +88,6 @@ struct FvArgs {
   int debug_no_issue;
   DevParams P;
 };
-
-// The stage's arithmetic constants as register values.  On GB300 an FP64 FMA whose operands
-// are all registers issues at 2.0 per clock per SM, while DADD, DMUL and any FP64 instruction
-// with a constant-bank operand (a kernel parameter or a literal) issue at 1.68 (measured), so
-// the constants that the adds, subtractions and products written as FMAs use (1, -1, 0, 1/2)
-// and the gas constants are copied into registers once per thread: a shuffle hides their
-// values from the compiler, which would otherwise fold them back into constant-bank operands.
-__device__ __forceinline__ double opaque_reg(double v) { return __shfl_sync(0xffffffffu, v, 0); }
-__device__ __forceinline__ FvArgs with_reg_params(const FvArgs& A) {
-  FvArgs L = A;
-  L.P.one = opaque_reg(A.P.one);
-  L.P.mone = opaque_reg(A.P.mone);
-  L.P.zero = opaque_reg(A.P.zero);
-  L.P.half = opaque_reg(A.P.half);
-  L.P.gamma = opaque_reg(A.P.gamma);
-  L.P.gm1 = opaque_reg(A.P.gm1);
-  L.P.Gamma = opaque_reg(A.P.Gamma);
-  L.P.Gq = opaque_reg(A.P.Gq);
-  return L;
-}
 
 // Tensor maps of the TMA-staged variant, per arena level of back-to-back patches: boxes of
 // one z-plane of a 16x16 or 32x8 column and of its four ring strips (x strips two voxels
@@ -182,16 +161,6 @@ __device__ __forceinline__ void derive(const FvArgs& A, int64_t e, const double*
   } else {
     PDE::prims(q, A.P, W);
   }
-}
-
-// f(integral_constant<int, 0>), f(integral_constant<int, 1>), ..: a loop whose index is a constant.
-template <class F, int... I>
-__device__ __forceinline__ void for_seq(F f, std::integer_sequence<int, I...>) {
-  (f(std::integral_constant<int, I>{}), ...);
-}
-template <int N, class F>
-__device__ __forceinline__ void for_n(F f) {
-  for_seq(f, std::make_integer_sequence<int, N>{});
 }
 
 // Systems whose derived quantities are many (SRHD: eight) form all three

@@ -9,10 +9,21 @@
 #pragma once
 
 #include <type_traits>
+#include <utility>
 
 #include "dh_internal.cuh"
 
 namespace dh {
+
+// f(integral_constant<int, 0>), f(integral_constant<int, 1>), ..: a loop whose index is a constant.
+template <class F, int... I>
+__device__ __forceinline__ void for_seq(F f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void for_n(F f) {
+  for_seq(f, std::make_integer_sequence<int, N>{});
+}
 
 __device__ __forceinline__ double sel3(int d, double a, double b, double c) {
   return d == 0 ? a : (d == 1 ? b : c);
@@ -32,6 +43,25 @@ __device__ __forceinline__ double sel3(int d, double a, double b, double c) {
 __device__ __forceinline__ double ADD(const DevParams& P, double a, double b) { return fma(a, P.one, b); }
 __device__ __forceinline__ double SUB(const DevParams& P, double a, double b) { return fma(b, P.mone, a); }
 __device__ __forceinline__ double MUL(const DevParams& P, double a, double b) { return fma(a, b, P.zero); }
+
+// The kernels' arithmetic constants as register values: the constants that the adds, subtractions and
+// products written as FMAs use and the gas constants are copied into registers once per thread; a
+// shuffle hides their values from the compiler, which would otherwise fold them back into constant-bank
+// operands.
+__device__ __forceinline__ double opaque_reg(double v) { return __shfl_sync(0xffffffffu, v, 0); }
+template <class Args>
+__device__ __forceinline__ Args with_reg_params(const Args& A) {
+  Args L = A;
+  L.P.one = opaque_reg(A.P.one);
+  L.P.mone = opaque_reg(A.P.mone);
+  L.P.zero = opaque_reg(A.P.zero);
+  L.P.half = opaque_reg(A.P.half);
+  L.P.gamma = opaque_reg(A.P.gamma);
+  L.P.gm1 = opaque_reg(A.P.gm1);
+  L.P.Gamma = opaque_reg(A.P.Gamma);
+  L.P.Gq = opaque_reg(A.P.Gq);
+  return L;
+}
 
 // 1/a for a normal, finite, positive or negative a: the hardware reciprocal
 // estimate y (PTX rcp.approx.ftz.f64, relative error below 2^-19.9 over 2^28
@@ -102,6 +132,11 @@ struct PdeAdvFlux {
   static constexpr bool FLUX = true, NCP = false, SRC = false, HYDRO = false;
   __device__ static constexpr bool moves(int) { return true; }
   __device__ static double vel(int d, const double* q, const double*) { return sel3(d, q[1], q[2], q[3]); }
+  __device__ static void edge(int d, const double* q, const DevParams&, double& u, double& p, double& lam) {
+    u = sel3(d, q[1], q[2], q[3]);
+    p = 0.0;
+    lam = fabs(u);
+  }
   __device__ static void prims(const double*, const DevParams&, double*) {}
   __device__ static void flux(int d, const double* q, const double*, const DevParams& P, double* F) {
     F[0] = MUL(P, sel3(d, q[1], q[2], q[3]), q[0]);
@@ -165,6 +200,17 @@ struct PdeEuler {
 #pragma unroll
     for (int v = 0; v < N; ++v) F[v] = v == 1 + d ? fma(q[v], u, p) : MUL(P, q[v], u);
     F[N - 1] = MUL(P, ADD(P, q[N - 1], p), u);
+  }
+  // Velocity, pressure and speed along d of a state whose other velocities are not needed (18 FP64
+  // operations).
+  __device__ static void edge(int d, const double* q, const DevParams& P, double& u, double& p, double& lam) {
+    const double r = recip_nr(q[0]);
+    double m2 = MUL(P, q[1], q[1]);
+#pragma unroll
+    for (int k = 1; k < DIM; ++k) m2 = fma(q[1 + k], q[1 + k], m2);
+    u = MUL(P, (DIM == 3) ? sel3(d, q[1], q[2], q[DIM == 3 ? 3 : 1]) : (d == 0 ? q[1] : q[2]), r);
+    p = MUL(P, P.gm1, fma(-P.half, MUL(P, m2, r), q[DIM + 1]));
+    lam = ADD(P, fabs(u), sqrt_pos(MUL(P, MUL(P, P.gamma, p), r)));
   }
   __device__ static double speed(int d, const double*, const double* w, const DevParams& P) {
     return ADD(P, fabs(vel(d, nullptr, w)), w[DIM + 1]);

@@ -15,8 +15,7 @@
 //             x z-march of whole patches or chunks of <= 16 planes
 //             x loads: plain (L2-prefetched) or, for 3D Euler, TMA tensor copies of every
 //               column plane and its ring strips into a double-buffered shared ring
-//   second-order FV stage: z-march of whole patches or in chunks of <= 16 planes, or the 8x8x4
-//             tile kernel;
+//   second-order FV stage: one form (the three values of its variant run the same tiles);
 //   FD stage: register cap (3 or 2 CTAs per SM) x staging (asynchronous copies or TMA);
 //             with TMA staging (systems of <= 5 variables) also caps for 3 and 4 CTAs per SM
 #include <cstdio>
