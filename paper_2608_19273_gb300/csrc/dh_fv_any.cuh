@@ -20,7 +20,8 @@
 // and direction; 71.7 KB for the Euler equations in 3D, three CTAs per SM.
 // Bound by the FP64 pipe: about 81 instructions a voxel, 144 when every line cell's flux was formed (the
 // face halo of a 6^3 box is as many cells as the box), direction after direction with two barriers
-// each, and every face sum was FP64.  16,384 patches of 6^3, two SSP-RK3 steps: 6.71 -> 4.97 ms (the FP64
+// each, and every face sum was FP64; a box whose W is at hand is copied asynchronously, all of it in flight
+// at once (4.97 ms with loads cell after cell).  16,384 patches of 6^3, two SSP-RK3 steps: 6.71 -> 4.61 ms (the FP64
 // instructions alone: 3.4); 4096 of 3^3: 0.23 ms.
 #pragma once
 
@@ -81,15 +82,38 @@ struct FvAny {
       sc[2] = A.d * dt * sc[0];
     }
 
+    // this voxel's element; what its update reads of the earlier stages is brought into L2 meanwhile
+    int64_t e = 0;
+    if (act) {
+      int k, x, y, z;
+      if (w.mp > 0) {
+        const int mx = lx >= w.mp, my = ly >= w.mp, mz = lz >= w.mp;
+        k = __ldg(w.patch + mx + 2 * my + 4 * mz);
+        x = lx - mx * w.mp; y = ly - my * w.mp; z = lz - mz * w.mp;
+      } else {
+        k = __ldg(w.patch + g);
+        x = w.x0 + lx; y = w.y0 + ly; z = DIM == 3 ? w.z0 + lz : 0;
+      }
+      const int pk = w.mp > 0 ? w.mp : p;
+      e = A.patches[k].offset + ((int64_t)z * pk + y) * pk + x;
+#pragma unroll
+      for (int v = 0; v < N; ++v) {
+        if (A.q0) prefetch_l2(A.q0 + v * A.vs + e);
+        if (A.acc && A.form != 1) prefetch_l2(A.acc + v * A.vs + e);
+      }
+    }
+
     // 1. the box and its face halo, with W: the cells that are read, enumerated group by group as
     //    the box (x fastest), then the two halo layers across x, y and z (edges and corners are
     //    never read and never visited)
     const int HX = by * bz, HY = bx * bz, HZ = DIM == 3 ? bx * by : 0;
     const int CG = nvg + 2 * (HX + HY + HZ);  // cells read per group
     const ADiv dCG(CG), dBX(bx), dBXY(bx * by), dBY(by), dHX(HX), dHY(HY), dHZ(HZ > 0 ? HZ : 1);
-    for (int j = tid; j < ng * CG; j += ANY_NT) {
+    // slot, arena element and halo direction of the j-th cell that is read
+    auto cell = [&](int j, int& s, int64_t& e, int& hd) {
       const int gg = dCG.q(j);
-      int r = j - gg * CG, cx, cy, cz, hd = -1;  // hd: the halo cell's direction
+      int r = j - gg * CG, cx, cy, cz;
+      hd = -1;  // a halo cell's direction
       if (r < nvg) {
         cz = DIM == 3 ? dBXY.q(r) : 0;
         const int rxy = r - cz * bx * by;
@@ -115,8 +139,7 @@ struct FvAny {
         cy = dBX.q(t);
         cx = t - cy * bx;
       }
-      const int s = gg * SG + ((DIM == 3 ? cz + 1 : 0) * SY + (cy + 1)) * SX + (cx + 1);
-      int64_t e;
+      s = gg * SG + ((DIM == 3 ? cz + 1 : 0) * SY + (cy + 1)) * SX + (cx + 1);
       if (w.mp > 0) {
         // a 2x2x2 block of mp^3 patches: the member holding the cell, and the cell's
         // coordinates in it (at most one outside [0, mp): a face neighbour of that member)
@@ -126,28 +149,56 @@ struct FvAny {
       } else {
         e = vox_index(A.patches, nullptr, __ldg(w.patch + gg), p, w.x0 + cx, w.y0 + cy, DIM == 3 ? w.z0 + cz : 0);
       }
-      double q[NV], W[NW];
+    };
+    if constexpr ((WM & 1) && PDE::M == 0) {
+      // the state and its W are copied as they are (velocity, pressure and sound speed lie in the
+      // order of W), asynchronously: every copy of the item is in flight at once
+      static_assert(NC == N + NW, "velocity, pressure and sound speed are W");
 #pragma unroll
-      for (int v = 0; v < N; ++v) q[v] = __ldg(A.qs + v * A.vs + e);
+      for (int it = 0; it < ANY_SLOTS / ANY_NT; ++it) {
+        const int j = tid + it * ANY_NT;
+        if (j < ng * CG) {
+          int s, hd;
+          int64_t e;
+          cell(j, s, e, hd);
 #pragma unroll
-      for (int v = 0; v < PDE::M; ++v) q[N + v] = __ldg(A.mat + v * A.vs + e);
-      if (WM & 1) {
-#pragma unroll
-        for (int i = 0; i < NW; ++i) W[i] = __ldg(A.w_in + i * A.vs + e);
-      } else {
-        PDE::prims(q, P, W);
+          for (int v = 0; v < NC; ++v) {
+            const double* src = v < N ? A.qs + v * A.vs + e : A.w_in + (v - N) * A.vs + e;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(Q + v * ANY_SLOTS + s)),
+                         "l"(src)
+                         : "memory");
+          }
+        }
       }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+    } else {
+      for (int j = tid; j < ng * CG; j += ANY_NT) {
+        int s, hd;
+        int64_t e;
+        cell(j, s, e, hd);
+        double q[NV], W[NW];
 #pragma unroll
-      for (int v = 0; v < N; ++v) Q[v * ANY_SLOTS + s] = q[v];
+        for (int v = 0; v < N; ++v) q[v] = __ldg(A.qs + v * A.vs + e);
 #pragma unroll
-      for (int d = 0; d < DIM; ++d) U[d * ANY_SLOTS + s] = PDE::vel(d, q, W);
-      if constexpr (HYDRO) Pr[s] = PDE::press(W);
-      if constexpr (SRHD) {
+        for (int v = 0; v < PDE::M; ++v) q[N + v] = __ldg(A.mat + v * A.vs + e);
+        if (WM & 1) {
 #pragma unroll
-        for (int d = 0; d < DIM; ++d)
-          if (hd < 0 || hd == d) L[d * ANY_SLOTS + s] = PDE::speed(d, q, W, P);
-      } else if constexpr (HYDRO) {
-        L[s] = W[DIM + 1];
+          for (int i = 0; i < NW; ++i) W[i] = __ldg(A.w_in + i * A.vs + e);
+        } else {
+          PDE::prims(q, P, W);
+        }
+#pragma unroll
+        for (int v = 0; v < N; ++v) Q[v * ANY_SLOTS + s] = q[v];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) U[d * ANY_SLOTS + s] = PDE::vel(d, q, W);
+        if constexpr (HYDRO) Pr[s] = PDE::press(W);
+        if constexpr (SRHD) {
+#pragma unroll
+          for (int d = 0; d < DIM; ++d)
+            if (hd < 0 || hd == d) L[d * ANY_SLOTS + s] = PDE::speed(d, q, W, P);
+        } else if constexpr (HYDRO) {
+          L[s] = W[DIM + 1];
+        }
       }
     }
     __syncthreads();
@@ -170,7 +221,7 @@ struct FvAny {
 #pragma unroll
         for (int v = 0; v < N; ++v) { qL[v] = Q[v * ANY_SLOTS + cLf]; qR[v] = Q[v * ANY_SLOTS + cR]; }
         const double uL = U[d * ANY_SLOTS + cLf], uR = U[d * ANY_SLOTS + cR];
-        double lL = fabs(uL), lR = fabs(uR);
+        double lL = abs_int(uL), lR = abs_int(uR);
         if constexpr (SRHD) { lL = L[d * ANY_SLOTS + cLf]; lR = L[d * ANY_SLOTS + cR]; }
         else if constexpr (HYDRO) { lL = ADD(P, lL, L[cLf]); lR = ADD(P, lR, L[cR]); }
         rusanov<PDE>(P, qL, uL, lL, qR, uR, lR, h);
@@ -192,19 +243,8 @@ struct FvAny {
 
     // 3. stage combination, W and lambda of the result
     if (!act) return;
-    int k, x, y, z;
-    if (w.mp > 0) {
-      const int mx = lx >= w.mp, my = ly >= w.mp, mz = lz >= w.mp;
-      k = __ldg(w.patch + mx + 2 * my + 4 * mz);
-      x = lx - mx * w.mp; y = ly - my * w.mp; z = lz - mz * w.mp;
-    } else {
-      k = __ldg(w.patch + g);
-      x = w.x0 + lx; y = w.y0 + ly; z = DIM == 3 ? w.z0 + lz : 0;
-    }
     const double cS = sc[1], cA = sc[2];
     const bool b1 = A.b == 1.0;
-    const int pk = w.mp > 0 ? w.mp : p;
-    const int64_t e = A.patches[k].offset + ((int64_t)z * pk + y) * pk + x;
     const int me = g * SG + ((DIM == 3 ? lz + 1 : 0) * SY + (ly + 1)) * SX + (lx + 1);
     double Qk[NV], res[NV];
 #pragma unroll

@@ -117,6 +117,14 @@ __device__ __forceinline__ double sqrt_pos(double x) {
   return sqrt(x);
 }
 
+// |a| by clearing the sign bit on the integer pipe (fabs as an operand of an FMA is an FP64
+// operation of its own).
+__device__ __forceinline__ double abs_int(double a) {
+  int h;
+  asm("and.b32 %0, %1, 0x7fffffff;" : "=r"(h) : "r"(__double2hiint(a)));
+  return __hiloint2double(h, __double2loint(a));
+}
+
 // max(a, b) for a, b >= +0 (characteristic speeds): non-negative doubles order
 // like their bit patterns read as signed 64-bit integers, so the comparison
 // runs on the integer pipe instead of the FP64 pipe.
@@ -210,10 +218,10 @@ struct PdeEuler {
     for (int k = 1; k < DIM; ++k) m2 = fma(q[1 + k], q[1 + k], m2);
     u = MUL(P, (DIM == 3) ? sel3(d, q[1], q[2], q[DIM == 3 ? 3 : 1]) : (d == 0 ? q[1] : q[2]), r);
     p = MUL(P, P.gm1, fma(-P.half, MUL(P, m2, r), q[DIM + 1]));
-    lam = ADD(P, fabs(u), sqrt_pos(MUL(P, MUL(P, P.gamma, p), r)));
+    lam = ADD(P, abs_int(u), sqrt_pos(MUL(P, MUL(P, P.gamma, p), r)));
   }
   __device__ static double speed(int d, const double*, const double* w, const DevParams& P) {
-    return ADD(P, fabs(vel(d, nullptr, w)), w[DIM + 1]);
+    return ADD(P, abs_int(vel(d, nullptr, w)), w[DIM + 1]);
   }
   __device__ static void ncp(int, const double*, const double*, const DevParams&, double*) {}
   __device__ static void source(const double*, const double*, const DevParams&, double*) {}
@@ -261,7 +269,7 @@ struct PdeSRHD {
   __device__ static double speed(int d, const double*, const double* w, const DevParams& P) {
     const double v = sel3(d, w[0], w[1], w[2]), omc = w[4];
     const double disc = MUL(P, w[5], fma(-MUL(P, v, v), omc, w[6]));
-    return MUL(P, fma(fabs(v), omc, sqrt_pos(disc)), w[7]);
+    return MUL(P, fma(abs_int(v), omc, sqrt_pos(disc)), w[7]);
   }
   // The largest speed over the three directions.  For |v_d| < 1 (and cs^2 < 1) the speed
   // increases with |v_d|:
