@@ -44,7 +44,7 @@ __device__ __forceinline__ double warp_max_d(double v) {
   return v;
 }
 
-// One CTA per patch: lambda of every voxel, block max, atomicMax on the bit
+// gridDim.y CTAs per patch (dh_plan::voxel_grid): lambda of every voxel, block max, atomicMax on the bit
 // pattern, last CTA publishes and resets the scratch.
 template <class PDE>
 __global__ void __launch_bounds__(256) k_max_speed(const dh_patch* __restrict__ patches, int dim, int64_t vs,
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256) k_max_speed(const dh_patch* __restrict__ 
   const dh_patch pt = patches[blockIdx.x];
   const int n = dim == 3 ? pt.p * pt.p * pt.p : pt.p * pt.p;
   double lam = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
     double u[PDE::N + PDE::M], W[PDE::NW > 0 ? PDE::NW : 1];
     const int64_t e = pt.offset + i;
 #pragma unroll
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256) k_max_speed(const dh_patch* __restrict__ 
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, wmax[i]);
     atomicMax(red, (unsigned long long)__double_as_longlong(m));
     __threadfence();
-    last = atomicAdd(red + 1, 1ull) == gridDim.x - 1;
+    last = atomicAdd(red + 1, 1ull) == (unsigned long long)gridDim.x * gridDim.y - 1;
   }
   __syncthreads();
   if (last && threadIdx.x == 0) {
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) k_max_speed_w(const dh_patch* __restrict_
   const dh_patch pt = patches[blockIdx.x];
   const int n = dim == 3 ? pt.p * pt.p * pt.p : pt.p * pt.p;
   double lam = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
     double W[PDE::NW];
     const int64_t e = pt.offset + i;
 #pragma unroll
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k_max_speed_w(const dh_patch* __restrict_
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, wmax[i]);
     atomicMax(red, (unsigned long long)__double_as_longlong(m));
     __threadfence();
-    last = atomicAdd(red + 1, 1ull) == gridDim.x - 1;
+    last = atomicAdd(red + 1, 1ull) == (unsigned long long)gridDim.x * gridDim.y - 1;
   }
   __syncthreads();
   if (last && threadIdx.x == 0) {
@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(256) k_max_speed_w(const dh_patch* __restrict_
 dh_status max_wave_speed_w(dh_plan* plan, const double* w, double* lam_out_dev, cudaStream_t s) {
   const dh_patch* P = plan->d_patches;
   switch (plan->pde) {
-    case DH_PDE_EULER2D: k_max_speed_w<PdeEuler2><<<plan->K, 256, 0, s>>>(P, 2, plan->var_stride, w, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_EULER3D: k_max_speed_w<PdeEuler3><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, w, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_EULER2D: k_max_speed_w<PdeEuler2><<<plan->voxel_grid(), 256, 0, s>>>(P, 2, plan->var_stride, w, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_EULER3D: k_max_speed_w<PdeEuler3><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, w, plan->params, lam_out_dev, plan->d_red); break;
     default:
       set_error("max_wave_speed_w: PDE %d keeps no derived quantities", plan->pde);
       return DH_EUNSUPPORTED;
@@ -145,7 +145,7 @@ __global__ void k_prim2con_euler(const dh_patch* __restrict__ patches, int64_t v
                                  double* __restrict__ q, double gamma) {
   const dh_patch pt = patches[blockIdx.x];
   const int n = DIM == 3 ? pt.p * pt.p * pt.p : pt.p * pt.p;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
     const int64_t e = pt.offset + i;
     const double rho = w[e], p = w[(DIM + 1) * vs + e];
     double kin = 0.0;
@@ -165,7 +165,7 @@ __global__ void k_prim2con_srhd(const dh_patch* __restrict__ patches, int64_t vs
                                 double* __restrict__ q, double G) {
   const dh_patch pt = patches[blockIdx.x];
   const int n = pt.p * pt.p * pt.p;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
     const int64_t e = pt.offset + i;
     const double rho = w[e], vx = w[vs + e], vy = w[2 * vs + e], vz = w[3 * vs + e], p = w[4 * vs + e];
     const double v2 = fma(vx, vx, fma(vy, vy, vz * vz));
@@ -502,6 +502,8 @@ dh_status dh_plan_create(dh_plan** out, int32_t pde, int32_t dim, const dh_patch
     plan->fv_var = pde == DH_PDE_SRHD3D && by16 && plan->n_wl[1] > 2 * n_sm ? 2 : 2 | (3 << 3);
   }
 
+  for (int k = 0; k < K; ++k) plan->max_p = std::max(plan->max_p, (int)patches[k].p);
+
   // FD tiles: 8x8x4 blocks (p is a multiple of 8)
   std::vector<FdWork> fdw;
   if (dim == 3 && !generic) {
@@ -679,13 +681,13 @@ dh_status max_wave_speed(dh_plan* plan, const double* q, const double* mat, doub
   cudaStream_t s = (cudaStream_t)stream;
   const dh_patch* P = plan->d_patches;
   switch (plan->pde) {
-    case DH_PDE_ADV_FLUX: k_max_speed<PdeAdvFlux><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_ADV_NCP: k_max_speed<PdeAdvNcp><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_EULER2D: k_max_speed<PdeEuler2><<<plan->K, 256, 0, s>>>(P, 2, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_EULER3D: k_max_speed<PdeEuler3><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_SRHD3D: k_max_speed<PdeSRHD><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_WAVE3D: k_max_speed<PdeWave><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
-    case DH_PDE_GW59: k_max_speed<PdeGW59><<<plan->K, 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_ADV_FLUX: k_max_speed<PdeAdvFlux><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_ADV_NCP: k_max_speed<PdeAdvNcp><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_EULER2D: k_max_speed<PdeEuler2><<<plan->voxel_grid(), 256, 0, s>>>(P, 2, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_EULER3D: k_max_speed<PdeEuler3><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_SRHD3D: k_max_speed<PdeSRHD><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_WAVE3D: k_max_speed<PdeWave><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
+    case DH_PDE_GW59: k_max_speed<PdeGW59><<<plan->voxel_grid(), 256, 0, s>>>(P, 3, plan->var_stride, q, mat, plan->params, lam_out_dev, plan->d_red); break;
     default:
       set_error("max_wave_speed: PDE %d not supported yet", plan->pde);
       return DH_EUNSUPPORTED;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -145,6 +146,17 @@ struct dh_plan {
   static constexpr int NRED = 8;
   unsigned long long* d_red = nullptr;
   int num_sms = 0;
+  int max_p = 0;  // the largest patch
+  // Grid of the kernels that take a patch's voxels in blocks of 256 (k_con2prim_patches, k_max_speed):
+  // a CTA per patch and, while there are fewer than 32 CTAs per SM, more of them for each.  One CTA
+  // per patch left SMs idle where patches are few and large.  Wave speed, us, one CTA per patch against
+  // this: 4096 patches of 16^3 936 : 946, 64 of 32^3 279 : 136, 8 of 64^3 2183 : 136, 8 of 16^3 41 : 9;
+  // the recovery gains alike (8 of 64^3 6088 : 279, its fewer FP64 operations included).
+  dim3 voxel_grid() const {
+    const long long n = dim == 3 ? 1ll * max_p * max_p * max_p : 1ll * max_p * max_p;
+    const long long y = (n + 255) / 256, cap = (32ll * num_sms + K - 1) / K;
+    return dim3((unsigned)K, (unsigned)std::max(1ll, std::min(std::min(y, cap), 65535ll)));
+  }
   // set by the runtime around the last FV stage of a time step whose successor's dt that
   // stage computes in its lambda epilogue (multi-step sequences), NULL otherwise
   double* dt_fold = nullptr;
