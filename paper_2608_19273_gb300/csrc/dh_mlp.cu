@@ -89,6 +89,7 @@ __global__ void k_mlp_forward(const float* __restrict__ wg, const float* __restr
 constexpr int GT = 256;   // threads of a gradient CTA
 constexpr int GP = 36;    // pitch of the per-sample rows (16-byte aligned, four banks further per sample)
 constexpr size_t GRAD_SMEM = sizeof(float) * (MLP_LEN + 32 * GP + 4 * GB * GP + 6 * GB);
+static_assert(GRAD_SMEM <= 48 * 1024, "within the default shared memory of a CTA");
 
 // Per-CTA partial gradient of (1/B) sum (y_i - t_i)^2 over samples [off, off + B).
 // part row layout: 1217 gradient entries, then the partial sum of squared residuals.
@@ -305,14 +306,6 @@ static AdamArgs adam_args(float* w, float* m, float* v, int32_t t, float lr, flo
 static dh_status grad_launch(const float* w, const float* x, const float* t, int64_t offset, int32_t B, float* partials,
                              float* grad, const AdamArgs& A, float* loss_out, cudaStream_t s) {
   const int nb = (B + GB - 1) / GB;
-  static int configured_device = -1;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (configured_device != dev) {
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GRAD_SMEM);
-    if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(k_mlp_grad)");
-    configured_device = dev;
-  }
   k_mlp_grad<<<nb, GT, GRAD_SMEM, s>>>(w, x, t, offset, B, partials);
   k_mlp_reduce<<<(MLP_NW + 1 + 31) / 32, RED_T, 0, s>>>(partials, nb, B, grad, A, loss_out);
   return cuda_error(cudaGetLastError(), "dh_mlp_grad launch");
