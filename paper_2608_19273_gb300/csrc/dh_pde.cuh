@@ -125,6 +125,11 @@ __device__ __forceinline__ double abs_int(double a) {
   return __hiloint2double(h, __double2loint(a));
 }
 
+// Whether a is positive and within about 2^-500 and 2^500 (integer pipe).
+__device__ __forceinline__ bool mid_range(double a) {
+  return (unsigned)(__double2hiint(a) - (523 << 20)) <= (unsigned)(1000 << 20);
+}
+
 // max(a, b) for a, b >= +0 (characteristic speeds): non-negative doubles order
 // like their bit patterns read as signed 64-bit integers, so the comparison
 // runs on the integer pipe instead of the FP64 pipe.
@@ -140,6 +145,7 @@ struct PdeAdvFlux {
   static constexpr bool FLUX = true, NCP = false, SRC = false, HYDRO = false;
   __device__ static constexpr bool moves(int) { return true; }
   __device__ static double vel(int d, const double* q, const double*) { return sel3(d, q[1], q[2], q[3]); }
+  template <bool>
   __device__ static void edge(int d, const double* q, const DevParams&, double& u, double& p, double& lam) {
     u = sel3(d, q[1], q[2], q[3]);
     p = 0.0;
@@ -210,14 +216,17 @@ struct PdeEuler {
     F[N - 1] = MUL(P, ADD(P, q[N - 1], p), u);
   }
   // Velocity, pressure and speed along d of a state whose other velocities are not needed (18 FP64
-  // operations).
+  // operations).  The squares of the momenta stay in range while density and energy lie within
+  // 2^-500 and 2^500 (m^2 <= 2 rho E); WIDE forms the velocities first, as prims does.
+  template <bool WIDE>
   __device__ static void edge(int d, const double* q, const DevParams& P, double& u, double& p, double& lam) {
     const double r = recip_nr(q[0]);
-    double m2 = MUL(P, q[1], q[1]);
+    double kin = WIDE ? MUL(P, q[1], MUL(P, q[1], r)) : MUL(P, q[1], q[1]);
 #pragma unroll
-    for (int k = 1; k < DIM; ++k) m2 = fma(q[1 + k], q[1 + k], m2);
+    for (int k = 1; k < DIM; ++k) kin = fma(q[1 + k], WIDE ? MUL(P, q[1 + k], r) : q[1 + k], kin);
+    if (!WIDE) kin = MUL(P, kin, r);
     u = MUL(P, (DIM == 3) ? sel3(d, q[1], q[2], q[DIM == 3 ? 3 : 1]) : (d == 0 ? q[1] : q[2]), r);
-    p = MUL(P, P.gm1, fma(-P.half, MUL(P, m2, r), q[DIM + 1]));
+    p = MUL(P, P.gm1, fma(-P.half, kin, q[DIM + 1]));
     lam = ADD(P, abs_int(u), sqrt_pos(MUL(P, MUL(P, P.gamma, p), r)));
   }
   __device__ static double speed(int d, const double*, const double* w, const DevParams& P) {
