@@ -12,17 +12,17 @@
 // (2 lanes per clock and SM) was the bound of this stage when the stencils were FP64 sums: 23 operations
 // for the sixth differences of a variable and 3 per derivative, of 160 (wave) and 2400 (GW59) a
 // voxel.  They are now sums in 64-bit fixed point on the integer pipe (dh_fixed.cuh, fd_stencil),
-// which the FP64 operations of the products and of the update run beside: 39 and 948 FP64
-// instructions a voxel are left, a fifth of them conversions at a third of an FMA's cost.
+// which the FP64 operations of the products and of the update run beside: 19 and 627 FP64
+// adds, products and FMAs a voxel are left, and a conversion for every sum.
 // Each variable with the tile's three-voxel face halos (edges and corners are never read by the
 // axis-aligned stencils) is brought into a padded 14x14x10 box of shared memory by asynchronous
-// copies, several variables ahead of its use (FdRing), so one barrier per variable is all the
+// copies, several variables ahead of its use (FdRing), so one split barrier per variable is all the
 // waiting there is; halo voxels outside the patch come from the face neighbours.  A variable's
 // update is written after the next variable's staging: its chain of FP64 operations (64 clocks each)
 // is then issued among the integer operations of the next stencil.
-// Measured per RK4 step: the wave system on 8.4 M voxels 17.9 -> 4.4 ms (39% of the time the FP64
-// operations alone take, half of the issue slots; 0.9 ms would be the memory's), GW59 on
-// 3.9 M voxels 97 -> 30.5 ms (FP64 pipe: 70% busy).  With the sums in FP64 and every variable staged by plain
+// Measured per RK4 step: the wave system on 8.4 M voxels 17.9 -> 3.98 ms (the FP64
+// and the integer pipe each half busy; 0.9 ms would be the memory's), GW59 on
+// 3.9 M voxels 97 -> 27.8 ms (FP64 pipe: three quarters busy).  With the sums in FP64 and every variable staged by plain
 // loads: 12 and 75 ms at best.  Fixed point with the boxes loaded a group of five at a time: 5.7 and 36.9;
 // TMA copies of dense boxes (no padding, so every neighbour's address takes selects): 5.2 for the wave
 // system, kept as a variant for it.
@@ -271,7 +271,7 @@ __device__ __forceinline__ void tma_load5(void* dst, const TmaDesc* map, int c0,
 // Bounded wait for phase `parity` of `bar`: gives up after ~2^27 SM clocks
 // (about 65 ms) and returns false.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  const long long t0 = clock64();
+  long long t0 = 0;
   while (true) {
     uint32_t done;
     asm volatile(
@@ -280,6 +280,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     if (done) return true;
+    if (t0 == 0) t0 = clock64();
     if (clock64() - t0 > (1ll << 27)) return false;
   }
 }
@@ -321,19 +322,30 @@ __device__ bool tma_wait_all(const FdArgs& A, uint64_t* bar, uint32_t parity) {
 }
 
 // Ring of NB padded boxes, one variable each: while variable i is computed, the copies of the
-// next NB - 1 variables are in flight (asynchronous 8-byte copies global -> shared, one commit
+// next NB - 2 variables are in flight (asynchronous 8-byte copies global -> shared, one commit
 // group per variable; every thread copies the same four of the 1024 slots of every variable, so
-// their indexes are formed once per tile).  One barrier per variable.
+// their indexes are formed once per tile).  One barrier per variable, split in two: a warp arrives for
+// variable i + 1 when it begins variable i (its copies of i + 1 have landed, its reads of i - 1 are done) and
+// waits for the other warps' arrival only when it needs i + 1, so that warps may be a variable apart, some
+// in integer stencils while others issue FP64 updates.  The box that new copies overwrite is that
+// of variable i - 2.  With __syncthreads for every variable (all warps in the same phase, one variable more
+// in flight) an RK4 step took 30.6 ms against 27.8 (GW59) and 4.36 against 3.98 (wave system).
 static_assert(FNSLOT == 4 * FNT, "four slots per thread");
 template <int NB>
 struct FdRing {
+  static constexpr int AHEAD = NB - 2;  // variables issued ahead of the current one
   double* box;         // NB x FBOX doubles of shared memory
+  uint64_t* bars;      // two barriers of one arrival per warp, used in turn
+  unsigned int* err;
   const double* qs;
   int64_t vs, e[4];    // arena elements of this thread's slots within a variable
   int c[4];            // their slots in a box
   int centre;
 
-  __device__ __forceinline__ FdRing(const FdArgs& A, const FdWork& w, int p, double* smem) : box(smem), qs(A.qs), vs(A.vs) {
+  __device__ __forceinline__ FdRing(const FdArgs& A, const FdWork& w, int p, double* smem, uint64_t* b)
+      : box(smem), bars(b), err(A.err), qs(A.qs), vs(A.vs) {
+    if (threadIdx.x < 2) mbar_init(&bars[threadIdx.x], FNT / 32);
+    __syncthreads();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       int x, y, z;
@@ -356,11 +368,17 @@ struct FdRing {
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  // Waits for the oldest group but NB - 2: after the barrier variable i of the sequence is in its
-  // box and every thread has left the box of variable i - 1, which the next copies overwrite.
-  __device__ __forceinline__ void wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(NB - 2) : "memory");
-    __syncthreads();
+  // This warp is ready for variable i: its copies of it have landed (all groups but the NB - 3 after it).
+  __device__ __forceinline__ void ready(int i) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(NB - 3) : "memory");
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bars[i & 1])) : "memory");
+  }
+  // After this, variable i of the sequence is in its box and every warp has left the box of variable
+  // i - 2 (a bounded wait; every warp arrives for every variable, so it does not run out).
+  __device__ __forceinline__ void wait(int i) {
+    if (!mbar_wait(&bars[i & 1], (i >> 1) & 1)) atomicOr(err, 1u);
   }
   __device__ __forceinline__ BoxAcc acc(int b) const { return BoxAcc{box + b * FBOX + centre}; }
 };
@@ -518,14 +536,16 @@ __device__ void fd_tile_generic(const FdArgs& A, const FdWork& w, double* smem, 
     if (!tma_wait_all(A, &bars[0], 0)) return;
     fd_voxel_wave(A, [&](int) { return TmaAcc{smem, lx, ly, lz}; }, e, C, lam_thread);
   } else {
-    FdRing<NB> R(A, w, p, smem);
+    FdRing<NB> R(A, w, p, smem, bars);
     auto var = [](int i) { return i >= N ? -1 : (WAVE ? (i + 1) % N : i); };  // order of the variables
 #pragma unroll
-    for (int i = 0; i < NB - 1; ++i) R.issue(var(i), i);
+    for (int i = 0; i < R.AHEAD; ++i) R.issue(var(i), i);
     fd_scalars(A, pt.dx, &C);
+    R.ready(0);
     auto stage = [&](int i) {  // i-th variable of the order
-      R.wait();
-      R.issue(var(i + NB - 1), (i + NB - 1) % NB);
+      R.wait(i);
+      R.issue(var(i + R.AHEAD), (i + R.AHEAD) % NB);
+      R.ready(i + 1);
       return R.acc(i % NB);
     };
     if constexpr (WAVE) {
@@ -569,13 +589,13 @@ __device__ __forceinline__ void gw59_finish(const FdArgs& A, int64_t e, double g
 // Variables in the order lapse, shift x, y, z, then per field Pi, psi_x, psi_y, psi_z, phi: each is
 // read from its box once, while the next ones stream in.
 template <int NB>
-__device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, double& lam_thread) {
+__device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, uint64_t* bars, double& lam_thread) {
   const DevParams& P = A.P;
   const int64_t vs = A.vs;
   const dh_patch& pt = A.patches[w.patch];
   const int p = pt.p;
   __shared__ FdScalars C;
-  FdRing<NB> R(A, w, p, smem);
+  FdRing<NB> R(A, w, p, smem, bars);
   const int64_t e = R.e[0];
   auto var = [](int i) {  // i-th variable of the order
     if (i < 4) return 55 + i;
@@ -584,12 +604,15 @@ __device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, dou
     return 5 * a + (j == 4 ? 0 : j + 1);
   };
 #pragma unroll
-  for (int i = 0; i < NB - 1; ++i) R.issue(var(i), i);
+  for (int i = 0; i < R.AHEAD; ++i) R.issue(var(i), i);
   fd_scalars(A, pt.dx, &C);
-  int next = NB - 1, buf = 0;  // next variable of the order to issue, box of the current one
+  R.ready(0);
+  int cur = 0, buf = 0;  // current variable of the order, its box
   auto stage = [&]() {
-    R.wait();
-    R.issue(var(next++), buf == 0 ? NB - 1 : buf - 1);
+    R.wait(cur);
+    R.issue(var(cur + R.AHEAD), buf >= NB - R.AHEAD ? buf + R.AHEAD - NB : buf + R.AHEAD);
+    R.ready(cur + 1);
+    ++cur;
     const BoxAcc S = R.acc(buf);
     buf = buf == NB - 1 ? 0 : buf + 1;
     return S;
@@ -725,7 +748,7 @@ constexpr int fd_ring() {
 template <class PDE, int VAR>
 __global__ void __launch_bounds__(FNT, (fd_min_blocks<PDE, VAR>())) k_fd_stage(const __grid_constant__ FdArgs A) {
   extern __shared__ __align__(128) double fd_smem[];
-  __shared__ __align__(8) uint64_t bars[1];
+  __shared__ __align__(8) uint64_t bars[2];
   constexpr bool TMA = (VAR & 4) != 0;
   constexpr int NB = fd_ring<PDE, VAR>();
   const FdWork w = A.work[blockIdx.x];
@@ -740,7 +763,7 @@ __global__ void __launch_bounds__(FNT, (fd_min_blocks<PDE, VAR>())) k_fd_stage(c
     __syncthreads();
     fd_tile_generic<PDE, true, NB>(A, w, smem, bars, lam);
   } else if constexpr (PDE::N == 59) {
-    fd_tile_gw59<NB>(A, w, fd_smem, lam);
+    fd_tile_gw59<NB>(A, w, fd_smem, bars, lam);
   } else {
     fd_tile_generic<PDE, false, NB>(A, w, fd_smem, bars, lam);
   }
