@@ -271,7 +271,7 @@ __device__ __forceinline__ void tma_load5(void* dst, const TmaDesc* map, int c0,
 // Bounded wait for phase `parity` of `bar`: gives up after ~2^27 SM clocks
 // (about 65 ms) and returns false.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  long long t0 = 0;
+  const long long t0 = clock64();
   while (true) {
     uint32_t done;
     asm volatile(
@@ -280,7 +280,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     if (done) return true;
-    if (t0 == 0) t0 = clock64();
     if (clock64() - t0 > (1ll << 27)) return false;
   }
 }
@@ -376,9 +375,19 @@ struct FdRing {
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bars[i & 1])) : "memory");
   }
   // After this, variable i of the sequence is in its box and every warp has left the box of variable
-  // i - 2 (a bounded wait; every warp arrives for every variable, so it does not run out).
+  // i - 2.  Bounded by a number of tries, not by the clock, which runs on while a CTA is preempted;
+  // every warp arrives for every variable, so it does not run out.
   __device__ __forceinline__ void wait(int i) {
-    if (!mbar_wait(&bars[i & 1], (i >> 1) & 1)) atomicOr(err, 1u);
+    for (int n = 0; n < (1 << 20); ++n) {
+      uint32_t done;
+      asm volatile(
+          "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+          : "=r"(done)
+          : "r"(smem_u32(&bars[i & 1])), "r"((uint32_t)(i >> 1) & 1u)
+          : "memory");
+      if (done) return;
+    }
+    atomicOr(err, 1u);
   }
   __device__ __forceinline__ BoxAcc acc(int b) const { return BoxAcc{box + b * FBOX + centre}; }
 };

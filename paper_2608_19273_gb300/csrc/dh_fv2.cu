@@ -32,8 +32,8 @@
 //     of their three values, a small state beside a large one would lose its low bits.)
 //   * lambda_max of the result: warp shuffles, one atomicMax per CTA on the
 //     bit pattern, last CTA publishes (no spin waits).
-// One SSP-RK3 step of 2.6 M voxels: 5.83 -> 5.02 ms with the face values and the fixed-point sums (about
-// 280 FP64 instructions a voxel and stage, 386 before; the pipe is 75% busy).  A z-march of whole columns,
+// One SSP-RK3 step of 2.6 M voxels: 5.83 -> 4.90 ms with the face values and the fixed-point sums (305
+// FP64 instructions a voxel and stage, 386 before; the pipe is 85% busy).  A z-march of whole columns,
 // which needs no halo states along z, took 4% longer than the tiles before these (128 registers with
 // spills) and is gone.
 #include <algorithm>

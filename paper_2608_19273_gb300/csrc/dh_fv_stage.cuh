@@ -36,8 +36,8 @@
 //     quantity and no flux per cell (it was 12 for the fluxes of a voxel and 3 per quantity and face).
 //   * The sum over a voxel's faces and cell terms is formed in fixed point on the integer pipe
 //     (fx_sum): 6 to 13 terms per quantity cost one conversion, not as many FP64 additions.
-//   Euler in 3D issues 80 FP64 instructions a voxel and stage (117 before these two), with the pipe
-//   75-80% busy: 10.5 M voxels of the 8^3/16^3/32^3 mix, two SSP-RK3 steps, 15.2 -> 10.9 ms.  The pipe is still
+//   Euler in 3D issues 72 FP64 instructions and 5 conversions a voxel and stage (117 before these two), with
+//   the pipe 73-80% busy: 10.5 M voxels of the 8^3/16^3/32^3 mix, two SSP-RK3 steps, 15.2 -> 10.9 ms.  The pipe is still
 //   the bound; the integer one is a quarter busy.  Measured on the way: the two changes alone 12.0;
 //   the z face after the barrier (beside the sums) and the plane's loads before the in-plane
 //   faces 11.65; the earlier stages' sums and state loaded before the barrier 10.9.  24 warps an SM

@@ -72,7 +72,7 @@ struct Cand {
 static int tune_candidates(const dh_plan* plan, int scheme, Cand* cands) {
   int nc = 0;
   if (scheme == 2) {
-    // second-order FV: z-march of whole patches, z-march in chunks of <= 16 planes, 8x8x4 tiles
+    // second-order FV: the three values run the same 8x8x4 tiles
     for (int v = 0; v < 3; ++v) cands[nc++] = {v, plan->fv_zs, plan->fd_var};
     return nc;
   }
