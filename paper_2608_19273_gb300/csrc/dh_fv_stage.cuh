@@ -369,10 +369,13 @@ struct FvTile {
     const double dxk = A.patches[kk].dx;
     const int x = (act ? w.x0[g] : 0) + lx, y = (act ? w.y0[g] : 0) + ly;
     const int64_t off = act ? A.patches[k].offset : 0;
-    // the tile's scalars, formed by one thread (a division takes about nine FP64 operations): -1/(2 dx)
-    // (faces hold twice the flux), g dt and d dt times it, g dt, d dt; read after the first barrier
-    __shared__ double sc[5];
-    if (tid == 0) {
+    // the scalars of each column, formed by its first thread (a division takes about nine FP64
+    // operations): -1/(2 dx) (faces hold twice the flux), g dt and d dt times it, g dt, d dt; read after the
+    // first barrier.  One set per column: the four columns of a tile are put together by patch size
+    // alone and may belong to levels of different dx.
+    __shared__ double scal[G][5];
+    double* sc = scal[g];
+    if (lxy == 0) {
       const double dt = *A.dt_dev;
       sc[0] = -0.5 / dxk;
       sc[3] = A.g * dt;
