@@ -215,9 +215,9 @@ __device__ __forceinline__ Stencil fd_stencil_fp64(double c, const double (&x)[3
 // weights are small integers (192 by magnitude for the sixth differences: eight bits above the
 // significand, which leaves two guard bits).  About 300 integer instructions and one conversion
 // per sum instead of 23 FP64 operations and 3 per derivative: bound by the integer pipe, which the
-// FP64 operations of the terms run beside.  The error of the sixth differences is below that
-// of the FP64 sums, which round at partial sums of up to eight times the values and then weigh them
-// by 15.  DM: bit d for the derivative along d.
+// FP64 operations of the terms run beside.  The units that complemented terms lack are counted and
+// added back, so sums of terms that fit are exact: odd or linear data give sixth differences of
+// exactly 0, as in FP64.  DM: bit d for the derivative along d.
 template <int DM, class Acc>
 __device__ __forceinline__ Stencil fd_stencil(const Acc& S, int v) {
   constexpr int SH = 2;
@@ -235,19 +235,27 @@ __device__ __forceinline__ Stencil fd_stencil(const Acc& S, int v) {
   }
   if (!fx_ok(e)) return fd_stencil_fp64<DM>(c, x);
   long long s[3] = {0, 0, 0};  // S_1, S_2, S_3
+  int n[3] = {0, 0, 0};        // minus their complemented terms
   Stencil R{0.0, {0.0, 0.0, 0.0}};
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     long long m[6];
+    int g[6];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) m[i] = fx_align<SH>(x[d][i], e);
-    s[0] += m[2] + m[3];
-    s[1] += m[1] + m[4];
-    s[2] += m[0] + m[5];
-    if (DM & (1 << d)) R.d[d] = fx_value<SH>(((m[3] - m[2]) << 3) + (m[1] - m[4]), e);
+    for (int i = 0; i < 6; ++i) {
+      m[i] = fx_align<SH>(x[d][i], e);
+      g[i] = fx_neg(x[d][i]);
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      s[r] += m[2 - r] + m[3 + r];
+      n[r] += g[2 - r] + g[3 + r];
+    }
+    if (DM & (1 << d))
+      R.d[d] = fx_value<SH>(((m[3] - m[2]) << 3) + (m[1] - m[4]) - (((g[3] - g[2]) << 3) + (g[1] - g[4])), e);
   }
   const long long t = (s[2] - 6 * s[1]) + (15 * s[0] - 60 * fx_align<SH>(c, e));
-  R.ko = fx_value<SH>(t, e);
+  R.ko = fx_value<SH>(t - ((n[2] - 6 * n[1]) + (15 * n[0] - 60 * fx_neg(c))), e);
   return R;
 }
 

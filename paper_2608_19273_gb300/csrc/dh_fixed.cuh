@@ -13,8 +13,8 @@
 // A term loses only what lies below 2^-SH units in the last place of the largest term, where a
 // chain of FP64 additions rounds at every partial sum: the error is at most the number of terms
 // (by weight) times 2^-SH ulp of the largest term plus half an ulp of the result.
-// Negative terms are complemented bit by bit (-x - 1, one unit off -x, far below that bound),
-// so equal terms with weights that sum to zero cancel to exactly 0.
+// Negative terms are complemented bit by bit (-x - 1, one unit off -x); the callers count those units
+// and add them back, so that terms are cut towards zero and terms that fit are exact.
 // The caller checks fx_ok(e): terms that are infinite, NaN or so large or small that an exponent
 // could leave the normal range take the FP64 operations instead.
 #pragma once
@@ -28,6 +28,10 @@ __device__ __forceinline__ int fx_exp(double x) { return __double2hiint(x) & 0x7
 
 // Whether terms of largest exponent e (in place) can be summed: e in [80, 2030] (biased).
 __device__ __forceinline__ bool fx_ok(int e) { return (unsigned)(e - (80 << 20)) <= (unsigned)((2030 - 80) << 20); }
+
+// -1 for a term that fx_align complements, else 0: subtracting it from the aligned term adds the
+// unit back, so that terms that fit are exact and -x is aligned to minus what x is.
+__device__ __forceinline__ int fx_neg(double x) { return __double2hiint(x) >> 31; }
 
 // x in units of 2^(e - 1075 - SH), towards minus infinity (zeros and terms 2^-63 below e give 0
 // or -1; 0 < SH < 11).
@@ -80,12 +84,12 @@ __device__ __forceinline__ double fx_sum(const double (&p)[NP], const double (&m
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     t += fx_align<SH>(p[i], e);
-    neg -= __double2hiint(p[i]) >> 31;
+    neg -= fx_neg(p[i]);
   }
 #pragma unroll
   for (int i = 0; i < NM; ++i) {
     t -= fx_align<SH>(m[i], e);
-    neg += __double2hiint(m[i]) >> 31;
+    neg += fx_neg(m[i]);
   }
   return fx_value<SH>(t + neg, e);
 }
