@@ -20,12 +20,12 @@
 // waiting there is; halo voxels outside the patch come from the face neighbours.  A variable's
 // update is written after the next variable's staging: its chain of FP64 operations (64 clocks each)
 // is then issued among the integer operations of the next stencil.
-// Measured per RK4 step: the wave system on 8.4 M voxels 17.9 -> 3.98 ms (the FP64
-// and the integer pipe each half busy; 0.9 ms would be the memory's), GW59 on
-// 3.9 M voxels 97 -> 27.8 ms (FP64 pipe: three quarters busy).  With the sums in FP64 and every variable staged by plain
-// loads: 12 and 75 ms at best.  Fixed point with the boxes loaded a group of five at a time: 5.7 and 36.9;
-// TMA copies of dense boxes (no padding, so every neighbour's address takes selects): 5.2 for the wave
-// system, kept as a variant for it.
+// Measured per RK4 step: the wave system on 8.4 M voxels 17.9 -> 4.43 ms (0.9 ms would be the
+// memory's), GW59 on 3.9 M voxels 97 -> 29.0 ms.  With the sums in FP64 and every variable staged by plain
+// loads: 12 and 75 ms at best.  Against one alignment for all sums whatever its loss (two guard bits, derivatives
+// of steep fields short of up to all their bits): 4.05 and 27.4.  That form with the boxes loaded a group of five
+// at a time: 5.7 and 36.9; with TMA copies of dense boxes (no padding, so every neighbour's address takes
+// selects): 5.2 for the wave system, kept as a variant for it.
 // GW59 goes variable by variable (lapse and shift first, then the 11 scalar-wave fields), keeping
 // per voxel only the coupling quantities (alpha, beta, grad alpha, phi_b Pi_b, source sums) in registers.
 #include <cuda.h>
@@ -211,19 +211,36 @@ __device__ __forceinline__ Stencil fd_stencil_fp64(double c, const double (&x)[3
   return R;
 }
 
-// In fixed point (dh_fixed.cuh): the 19 values are aligned once and serve all four sums, whose
-// weights are small integers (192 by magnitude for the sixth differences: eight bits above the
-// significand, which leaves two guard bits).  About 300 integer instructions and one conversion
-// per sum instead of 23 FP64 operations and 3 per derivative: bound by the integer pipe, which the
-// FP64 operations of the terms run beside.  The units that complemented terms lack are counted and
-// added back, so sums of terms that fit are exact: odd or linear data give sixth differences of
-// exactly 0, as in FP64.  DM: bit d for the derivative along d.
-template <int DM, class Acc>
+// One unscaled derivative in FP64 operations, its values read again.  Not inlined: in GW59's nine
+// stencils the code for a few warps in a hundred took 0.6 ms of an RK4 step of 29.0 (3.9 M voxels).
+template <int D, class Acc>
+__device__ __noinline__ double fd_derivative(const Acc& S, int v) {
+  return fma(8.0, S.template nb<D>(v, 1) - S.template nb<D>(v, -1), S.template nb<D>(v, -2) - S.template nb<D>(v, 2));
+}
+
+// In fixed point (dh_fixed.cuh): the 19 values are aligned once, with five guard bits, and serve all
+// four sums, in integer instructions and one conversion per sum instead of 23 FP64 operations and 3 per
+// derivative: bound by the integer pipe, which the FP64 operations of the terms run beside.  The units that complemented terms lack are counted, so sums of terms that fit are exact
+// (odd or linear data give sixth differences of exactly 0, as in FP64).  The sixth differences are
+// T_3 - 6 T_2 + 15 T_1 with T_r = S_r - 6c, the grouping of the FP64 form: the T_r need four bits above the
+// terms and are exact sums; only where T_1 or T_2 is large are all three shifted by three bits to make
+// room for the weights (22 units of a quarter ulp of the largest value at most).
+// Terms far below the largest of the 19 lose bits.  For the sixth differences, which read all of them,
+// the error stays below that of the FP64 form; a derivative, which reads four, takes its three FP64
+// operations where both neighbours along its direction lie more than four binades below the largest
+// (a field steep along another direction: its four values may be the small ones).
+// Mean error, this over the FP64 form: smooth fields at 16 to 128 voxels a wave 0.00-0.09 (sixth differences)
+// and 0.62-0.95 (derivatives); a Gaussian pulse of 6.4 voxels 2, 8, 12 and 20 widths from its centre 0.00, 0.05,
+// 0.36, 0.83 and 0.94, 0.56, 0.84, 1.00; white noise 0.45 and 1.00.
+// DM: bit d for the derivative along d.  KEEP: the values stay in registers for the FP64 derivatives, which
+// in the tails of a pulse most voxels take (RK4 step of the wave system, 8.4 M voxels, nearly all
+// in the tails: 4.43 ms, 4.83 with calls of fd_derivative; GW59 without registers to spare 32.4 and 29.0).
+template <int DM, bool KEEP, class Acc>
 __device__ __forceinline__ Stencil fd_stencil(const Acc& S, int v) {
-  constexpr int SH = 2;
+  constexpr int SH = 5;
   double x[3][6];  // values at -3, -2, -1, +1, +2, +3
   const double c = S.val(v);
-  int e = fx_exp(c);
+  int e = fx_exp(c), nd[3];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     const int o = i < 3 ? i - 3 : i - 2;
@@ -231,9 +248,16 @@ __device__ __forceinline__ Stencil fd_stencil(const Acc& S, int v) {
     x[1][i] = S.template nb<1>(v, o);
     x[2][i] = S.template nb<2>(v, o);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) e = max(e, fx_exp(x[d][i]));
+    for (int d = 0; d < 3; ++d)
+      if (i != 2 && i != 3) e = max(e, fx_exp(x[d][i]));
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    nd[d] = max(fx_exp(x[d][2]), fx_exp(x[d][3]));
+    e = max(e, nd[d]);
   }
   if (!fx_ok(e)) return fd_stencil_fp64<DM>(c, x);
+  const int low = e - (4 << 20);
   long long s[3] = {0, 0, 0};  // S_1, S_2, S_3
   int n[3] = {0, 0, 0};        // minus their complemented terms
   Stencil R{0.0, {0.0, 0.0, 0.0}};
@@ -251,11 +275,38 @@ __device__ __forceinline__ Stencil fd_stencil(const Acc& S, int v) {
       s[r] += m[2 - r] + m[3 + r];
       n[r] += g[2 - r] + g[3 + r];
     }
-    if (DM & (1 << d))
-      R.d[d] = fx_value<SH>(((m[3] - m[2]) << 3) + (m[1] - m[4]) - (((g[3] - g[2]) << 3) + (g[1] - g[4])), e);
+    if (DM & (1 << d)) {
+      if (KEEP && nd[d] < low) R.d[d] = fma(8.0, x[d][3] - x[d][2], x[d][1] - x[d][4]);
+      else R.d[d] = fx_value<SH>(((m[3] - m[2]) << 3) + (m[1] - m[4]) - (((g[3] - g[2]) << 3) + (g[1] - g[4])), e);
+    }
   }
-  const long long t = (s[2] - 6 * s[1]) + (15 * s[0] - 60 * fx_align<SH>(c, e));
-  R.ko = fx_value<SH>(t - ((n[2] - 6 * n[1]) + (15 * n[0] - 60 * fx_neg(c))), e);
+  const long long c6 = 6 * fx_align<SH>(c, e);
+  const int n6 = 6 * fx_neg(c);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) s[r] -= c6;  // T_r, up to the units in n
+  int ek = e;
+  long long t;
+  if ((unsigned)((int)(s[0] >> 32) + (1 << 25)) >= (1u << 26) || (unsigned)((int)(s[1] >> 32) + (1 << 26)) >= (1u << 27)) {
+    // |T_1| >= 2^57 or |T_2| >= 2^58: 15 |T_1| + 6 |T_2| + |T_3| < 25.5 x 2^58 below these
+#pragma unroll
+    for (int r = 0; r < 3; ++r) s[r] = (s[r] - (n[r] - n6) + 4) >> 3;
+    t = (s[2] - 6 * s[1]) + 15 * s[0];
+    ek += 3 << 20;
+  } else {
+    t = (s[2] - 6 * s[1]) + 15 * s[0] - ((n[2] - 6 * n[1]) + (15 * n[0] - 10 * n6));
+  }
+  R.ko = fx_value<SH>(t, ek);
+  if constexpr (DM != 0 && !KEEP) {
+    int least = low;
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      if (DM & (1 << d)) least = min(least, nd[d]);
+    if (least < low) {
+      if ((DM & 1) && nd[0] < low) R.d[0] = fd_derivative<0>(S, v);
+      if ((DM & 2) && nd[1] < low) R.d[1] = fd_derivative<1>(S, v);
+      if ((DM & 4) && nd[2] < low) R.d[2] = fd_derivative<2>(S, v);
+    }
+  }
   return R;
 }
 
@@ -499,20 +550,20 @@ __device__ __forceinline__ void fd_voxel_wave(const FdArgs& A, Stage stage, int6
   {
     const auto S = stage(1);
     Pi = S.val(1);
-    sp = fd_stencil<7>(S, 1);
+    sp = fd_stencil<7, true>(S, 1);
   }
   const FdOld o2 = fd_old(A, 2 * vs + e);
   {
     const auto S = stage(2);
     q1 = S.val(2);
-    s1 = fd_stencil<1>(S, 2);
+    s1 = fd_stencil<1, true>(S, 2);
   }
   const FdOld o3 = fd_old(A, 3 * vs + e);
   {
     const auto S = stage(3);
     fd_combine(A, 2 * vs + e, o2, q1, fma(C.ko, s1.ko, PMUL(P, C.r12, sp.d[0])), C.gdt, C.ddt);
     q2 = S.val(3);
-    s2 = fd_stencil<2>(S, 3);
+    s2 = fd_stencil<2, true>(S, 3);
     div = PADD(P, s1.d[0], s2.d[1]);
   }
   const FdOld o4 = fd_old(A, 4 * vs + e);
@@ -520,7 +571,7 @@ __device__ __forceinline__ void fd_voxel_wave(const FdArgs& A, Stage stage, int6
     const auto S = stage(4);
     fd_combine(A, 3 * vs + e, o3, q2, fma(C.ko, s2.ko, PMUL(P, C.r12, sp.d[1])), C.gdt, C.ddt);
     q3 = S.val(4);
-    s3 = fd_stencil<4>(S, 4);
+    s3 = fd_stencil<4, true>(S, 4);
     div = PADD(P, div, s3.d[2]);
   }
   const FdOld o0 = fd_old(A, e);
@@ -528,7 +579,7 @@ __device__ __forceinline__ void fd_voxel_wave(const FdArgs& A, Stage stage, int6
     const auto S = stage(0);
     fd_combine(A, 4 * vs + e, o4, q3, fma(C.ko, s3.ko, PMUL(P, C.r12, sp.d[2])), C.gdt, C.ddt);
     fd_combine(A, vs + e, o1, Pi, fma(C.ko, sp.ko, fma(PMUL(P, PMUL(P, c, c), C.r12), div, PMUL(P, -P.damp, Pi))), C.gdt, C.ddt);
-    fd_combine(A, e, o0, S.val(0), fma(C.ko, fd_stencil<0>(S, 0).ko, Pi), C.gdt, C.ddt);
+    fd_combine(A, e, o0, S.val(0), fma(C.ko, fd_stencil<0, true>(S, 0).ko, Pi), C.gdt, C.ddt);
   }
   if (A.lam_out) lam_thread = fmax(lam_thread, c);
 }
@@ -575,7 +626,7 @@ __device__ void fd_tile_generic(const FdArgs& A, const FdWork& w, double* smem, 
       for (int v = 0; v < N; ++v) {
         const BoxAcc S = stage(v);
         q[v] = S.val(v);
-        const Stencil s = fd_stencil<7>(S, v);
+        const Stencil s = fd_stencil<7, true>(S, v);
         ko[v] = s.ko;
 #pragma unroll
         for (int d = 0; d < 3; ++d) dq[d][v] = PDE::needs_grad(d, v) ? PMUL(A.P, s.d[d], C.r12) : 0.0;
@@ -644,7 +695,7 @@ __device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, uin
     const BoxAcc S = stage();
     const double r12 = C.r12;
     G.al = S.val(0);
-    const Stencil s = fd_stencil<7>(S, 0);
+    const Stencil s = fd_stencil<7, false>(S, 0);
     G.dal0 = PMUL(P, s.d[0], r12);
     G.dal1 = PMUL(P, s.d[1], r12);
     G.dal2 = PMUL(P, s.d[2], r12);
@@ -657,7 +708,7 @@ __device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, uin
     const double b = S.val(0);
     (v == 1 ? G.bx : v == 2 ? G.by : G.bz) = b;
     (v == 1 ? G.bxr : v == 2 ? G.byr : G.bzr) = PMUL(P, b, C.r12);
-    G.ko_ab[v] = PMUL(P, C.ko, fd_stencil<0>(S, 0).ko);
+    G.ko_ab[v] = PMUL(P, C.ko, fd_stencil<0, false>(S, 0).ko);
   }
   const double ko = C.ko, gdt = C.gdt, ddt = C.ddt;
   const double al = G.al, bx = G.bx, by = G.by, bz = G.bz, alr = G.alr, bxr = G.bxr, byr = G.byr, bzr = G.bzr;
@@ -677,7 +728,7 @@ __device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, uin
       const BoxAcc S = stage();
       if (a > 0) fd_combine(A, eb - 5 * vs, op, phi, Lphi, gdt, ddt);
       Pi = S.val(0);
-      sP = fd_stencil<7>(S, 0);
+      sP = fd_stencil<7, false>(S, 0);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {  // psi_x, psi_y, psi_z, phi
@@ -705,11 +756,11 @@ __device__ void fd_tile_gw59(const FdArgs& A, const FdWork& w, double* smem, uin
         fd_combine(A, eb + vs, oP, Pi, fma(alr, div, LPi), gdt, ddt);
         phi = S.val(0);
         op = on;
-        Lphi = fma(ko, fd_stencil<0>(S, 0).ko, Lphi);
+        Lphi = fma(ko, fd_stencil<0, false>(S, 0).ko, Lphi);
       } else {
         ps = S.val(0);
         o = on;
-        s = fd_stencil<7>(S, 0);
+        s = fd_stencil<7, false>(S, 0);
       }
     }
   }
