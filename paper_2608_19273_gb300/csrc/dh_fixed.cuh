@@ -57,7 +57,9 @@ __device__ __forceinline__ double fx_value(long long t, int e) {
 
 // p[0] + .. + p[NP-1] - m[0] - .. - m[NM-1], with NP + NM <= 24 (five bits above the 53 + 5 of a
 // term): about 13 integer instructions per term and one conversion, instead of NP + NM - 1 FP64
-// additions.  With NP = NM and p[i] = m[i] the sum is exactly 0 in either form.
+// additions.  With NP = NM and p[i] = m[i] the sum is exactly 0 in either form.  A term that lies far
+// below the largest loses bits even where the largest ones cancel: where that can happen (the pressures
+// beside the momentum fluxes of a slow flow), the caller passes the difference as one term.
 template <int NP, int NM>
 __device__ __forceinline__ double fx_sum(const double (&p)[NP], const double (&m)[NM]) {
   static_assert(NP + NM <= 24 && NM <= NP, "room for the terms");

@@ -32,7 +32,7 @@
 //     of their three values, a small state beside a large one would lose its low bits.)
 //   * lambda_max of the result: warp shuffles, one atomicMax per CTA on the
 //     bit pattern, last CTA publishes (no spin waits).
-// One SSP-RK3 step of 2.6 M voxels: 5.83 -> 4.90 ms with the face values and the fixed-point sums (305
+// One SSP-RK3 step of 2.6 M voxels: 5.83 -> 4.92 ms with the face values and the fixed-point sums (308
 // FP64 instructions a voxel and stage, 386 before; the pipe is 85% busy).  A z-march of whole columns,
 // which needs no halo states along z, took 4% longer than the tiles before these (128 registers with
 // spills) and is gone.
@@ -272,14 +272,23 @@ struct Fv2Tile {
     double q[NV], res[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) q[v] = box[v * MBOX + me];
-#pragma unroll
-    for (int v = 0; v < N; ++v) {
+    for_n<N>([&](auto vc) {
+      constexpr int v = decltype(vc)::value;
       const int64_t ev = (int64_t)v * A.vs + e;
-      double tp[3], tm[3];
+      // the faces along a momentum's own direction hold the pressure: one term, so that nearly equal pressures
+      // far above the momentum cancel exactly (fx_sum)
+      constexpr int own = HYDRO && v >= 1 && v <= 3 ? v - 1 : -1;
+      double tp[3], tm[own >= 0 ? 2 : 3];
+      int n = 0;
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        tp[d] = H[(d * N + v) * MFS + fp[d]];
-        tm[d] = H[(d * N + v) * MFS + fm[d]];
+        const double hi = H[(d * N + v) * MFS + fp[d]], lo = H[(d * N + v) * MFS + fm[d]];
+        if (d == own) {
+          tp[2] = SUB(P, hi, lo);
+        } else {
+          tp[n] = hi;
+          tm[n++] = lo;
+        }
       }
       const double sum = fx_sum(tp, tm);
       if (A.out) {
@@ -293,7 +302,7 @@ struct Fv2Tile {
         if (!A.out) res[v] = r;
       }
       if (A.out) A.out[ev] = res[v];
-    }
+    });
     if (A.lam_out) {
 #pragma unroll
       for (int v = N; v < NV; ++v) res[v] = q[v];

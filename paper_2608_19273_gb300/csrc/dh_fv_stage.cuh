@@ -36,11 +36,13 @@
 //     quantity and no flux per cell (it was 12 for the fluxes of a voxel and 3 per quantity and face).
 //   * The sum over a voxel's faces and cell terms is formed in fixed point on the integer pipe
 //     (fx_sum): 6 to 13 terms per quantity cost one conversion, not as many FP64 additions.
-//   Euler in 3D issues 72 FP64 instructions and 5 conversions a voxel and stage (117 before these two), with
-//   the pipe 73-80% busy: 10.5 M voxels of the 8^3/16^3/32^3 mix, two SSP-RK3 steps, 15.2 -> 10.9 ms.  The pipe is still
+//     The pressures beside a voxel enter as one term, their difference: as two, they would cut the
+//     momentum fluxes of a slow flow at 2^-58 of the pressure even where they cancel (10.9 -> 11.06 ms below).
+//   Euler in 3D issues 75 FP64 instructions and 5 conversions a voxel and stage (117 before these two), with
+//   the pipe 73-80% busy: 10.5 M voxels of the 8^3/16^3/32^3 mix, two SSP-RK3 steps, 15.2 -> 11.06 ms.  The pipe is still
 //   the bound; the integer one is a quarter busy.  Measured on the way: the two changes alone 12.0;
 //   the z face after the barrier (beside the sums) and the plane's loads before the in-plane
-//   faces 11.65; the earlier stages' sums and state loaded before the barrier 10.9.  24 warps an SM
+//   faces 11.65; the earlier stages' sums and state loaded before the barrier 10.88.  24 warps an SM
 //   at 80 registers (spills): 12.9.
 //   * The maximum characteristic speed of the result is reduced with warp
 //     shuffles, then one atomicMax per CTA on the bit pattern (valid for
@@ -49,7 +51,6 @@
 
 #include <algorithm>
 #include <type_traits>
-
 
 #include "dh_fixed.cuh"
 #include "dh_internal.cuh"
@@ -574,16 +575,14 @@ struct FvTile {
           // cell terms of the neighbours (those of the voxel itself cancel), the raw sum R of the
           // earlier stages in the second stage of the stage-sum form
           constexpr bool MOM = HYDRO && v >= 1 && v <= DIM, EN = HYDRO && v == N - 1;
-          constexpr int NC = DIM + (MOM ? 1 : 0) + (EN ? DIM : 0);
-          constexpr int NPT = NC + (PDE::NCP ? 2 * DIM : 0) + 1;
+          constexpr int NC = DIM + (EN ? DIM : 0);
+          constexpr int NPT = NC + (MOM ? 1 : 0) + (PDE::NCP ? 2 * DIM : 0) + 1;
           double tp[NPT], tm[NC];
           tp[0] = S.Hx[v * FX + fxr]; tm[0] = S.Hx[v * FX + fxl];
           tp[1] = S.Hy[v * FY + fyu]; tm[1] = S.Hy[v * FY + fyl];
           if constexpr (DIM == 3) { tp[DIM - 1] = Hzhi[v]; tm[DIM - 1] = Hzlo[v]; }
-          if constexpr (MOM) {
-            tp[DIM] = v == 1 ? S.X[cxp] : v == 2 ? S.X[cyp] : pn;
-            tm[DIM] = v == 1 ? S.X[cxm] : v == 2 ? S.X[cym] : pm;
-          }
+          if constexpr (MOM)  // (one term, see fx_sum: nearly equal pressures far above the momentum cancel exactly)
+            tp[DIM] = SUB(P, v == 1 ? S.X[cxp] : v == 2 ? S.X[cyp] : pn, v == 1 ? S.X[cxm] : v == 2 ? S.X[cym] : pm);
           if constexpr (EN) {
             tp[DIM] = S.X[NXS + cxp]; tm[DIM] = S.X[NXS + cxm];
             tp[DIM + 1] = S.X[2 * NXS + cyp]; tm[DIM + 1] = S.X[2 * NXS + cym];

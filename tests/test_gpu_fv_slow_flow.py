@@ -77,3 +77,30 @@ def test_shear_under_uniform_pressure(kernel, mach, a):
         jump = (up - np.roll(sig, -1, b) / 2) - (L + sig / 2)  # of the upper face
         ref += np.longdouble(dt) / (2 * np.longdouble(dx)) * s * (jump - np.roll(jump, 1, b))
     assert np.max(np.abs(got - ref)) <= 16 * U * np.max(np.abs(m))
+
+
+@pytest.mark.parametrize("kernel", [k for k in KERNELS if k != "srhd"])
+def test_contact_at_rest_is_kept(kernel):
+    """A density that varies under a uniform pressure with no flow: only the density changes.  The energy's
+    face value Q_L (u_L + s) + Q_R (u_R - s) is there the rounding of E s, at most u E s, and with
+    dt s/dx <= 1/6 the six of a voxel move the energy by at most 6 x u E s x dt/(2 dx) <= u E/2, no more than
+    half a unit in its last place: the update rounds to the same energy, and the momentum stays exactly 0."""
+    torch = require_cuda()
+    pde, scheme, n, p, fv_var = KERNELS[kernel]
+    mesh = single_level(n, p, 2.0 ** -5)
+    N = n[0] * p
+    rho = np.random.default_rng(52).uniform(0.5, 1.5, (N, N, N))
+    q = np.zeros((5, N, N, N))
+    q[0], q[4] = rho, 2.6875
+    Q = np.stack([from_grid(mesh, np.ascontiguousarray(g), arena(mesh, 1)[0]) for g in q])
+    s_max = np.sqrt(1.4 * 0.4 * 2.6875 / rho.min())
+    with dh.Plan(pde, 3, mesh.patches, 2 if scheme == 2 else 1, mesh.var_stride) as plan:
+        if fv_var is not None:
+            dh.dh_plan_set_variant(plan, fv_var, 0, 0)
+        out = torch.zeros(Q.shape, dtype=torch.float64, device="cuda")
+        d_dt = torch.tensor([0.16 * 2.0 ** -5 / s_max], dtype=torch.float64, device="cuda")
+        f = dh.patch_update_fv_muscl if scheme == 2 else dh.patch_update_fv
+        f(plan, dev(torch, Q), None, out, None, None, d_dt, 0.0, 1.0, 1.0, 0.0)
+        got = np.stack([to_grid(mesh, g) for g in host(out)])
+    assert np.array_equal(got[1:], q[1:])
+    assert not np.array_equal(got[0], rho)
