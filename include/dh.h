@@ -397,8 +397,10 @@ dh_status dh_graph_stage_times(dh_plan* plan, float* ms_out, int32_t n);
  * `out` is overwritten.  If cache_path is NULL the environment variable
  * DH_TUNE_CACHE names the cache file (no cache when it is unset).  With a cache
  * file the choice is first looked up
- * there (one JSON object per line, keyed by GPU name, PDE, scheme and patch-size
- * histogram) and, when timed, appended to it.  choice_out (optional, 4 ints):
+ * there (one JSON object per line, keyed by GPU name, PDE, scheme, revision of
+ * the kernels, whether the plan takes TMA-staged variants and patch-size
+ * histogram; a choice that the plan refuses counts as not found) and, when timed,
+ * appended to it.  choice_out (optional, 4 ints):
  * fv_var, fv_zs, fd_var, 1 if taken from the cache.  times_out (optional,
  * DH_TUNE_MAX_CANDIDATES floats): ms per launch of each candidate, in the order
  * tile shape, grid, z-march, then fv_var bits 0-1 (unused entries untouched). */

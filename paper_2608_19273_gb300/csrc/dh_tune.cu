@@ -28,14 +28,26 @@
 
 namespace dh {
 
+static bool fv_tma_ok(const dh_plan* plan) {
+  return plan->pde == DH_PDE_EULER3D && plan->tma_ok && !plan->coupled && plan->n_lvl <= 8;
+}
+
+// Raised whenever a change of the kernels may change which of them is the fastest, so that choices saved
+// before it are timed again (2: sums in fixed point, the FD stage's ring of boxes).
+constexpr int TUNE_REVISION = 2;
+
+// What a saved choice holds for: GPU, PDE, scheme, dimension, revision of the kernels, whether the plan takes
+// the TMA-staged variants, patch sizes.
 static std::string tune_key(const dh_plan* plan, int scheme) {
   std::map<int, int> mix;
   for (const dh_patch& p : plan->h_patches) mix[p.p]++;
   cudaDeviceProp prop;
   std::string dev = "gpu";
   if (cudaGetDeviceProperties(&prop, plan->device) == cudaSuccess) dev = prop.name;
+  const bool tma = scheme == 0 ? fv_tma_ok(plan) : plan->tma_ok;
   std::string k = dev + "|pde=" + std::to_string(plan->pde) + "|scheme=" + std::to_string(scheme) +
-                  "|dim=" + std::to_string(plan->dim) + "|mix=";
+                  "|dim=" + std::to_string(plan->dim) + "|rev=" + std::to_string(TUNE_REVISION) +
+                  "|tma=" + std::to_string((int)tma) + "|mix=";
   for (auto& kv : mix) k += std::to_string(kv.first) + "x" + std::to_string(kv.second) + ",";
   return k;
 }
@@ -58,10 +70,6 @@ static bool cache_lookup(const char* path, const std::string& key, int* fv_var, 
   }
   fclose(f);
   return found;
-}
-
-static bool fv_tma_ok(const dh_plan* plan) {
-  return plan->pde == DH_PDE_EULER3D && plan->tma_ok && !plan->coupled && plan->n_lvl <= 8;
 }
 
 // The candidates of a plan (see the top of this file), in the order the timings are reported.
@@ -136,9 +144,12 @@ static dh_status tune_run(dh_plan* plan, int scheme, const std::string& key, int
   if (!cache_path) cache_path = std::getenv("DH_TUNE_CACHE");  // NULL and unset: no cache
   int v = 0, z = 0, f = 0;
   if (cache_path && cache_lookup(cache_path, key, &v, &z, &f)) {
-    dh_status st = scheme == 2 ? dh_plan_set_variant_muscl(plan, v) : dh_plan_set_variant(plan, v, z, f);
-    if (st == DH_OK && choice_out) { choice_out[0] = v; choice_out[1] = z; choice_out[2] = f; choice_out[3] = 1; }
-    return st;
+    // a choice that the plan refuses is timed anew
+    const dh_status st = scheme == 2 ? dh_plan_set_variant_muscl(plan, v) : dh_plan_set_variant(plan, v, z, f);
+    if (st == DH_OK) {
+      if (choice_out) { choice_out[0] = v; choice_out[1] = z; choice_out[2] = f; choice_out[3] = 1; }
+      return DH_OK;
+    }
   }
   Cand cands[DH_TUNE_MAX_CANDIDATES];
   const int nc = tune_candidates(plan, scheme, cands);
