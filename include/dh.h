@@ -389,11 +389,12 @@ dh_status dh_graph_stage_times(dh_plan* plan, float* ms_out, int32_t n);
  *                  x z-march in whole patches or in chunks of <= 16 planes;
  *                  the persistent grid and the 32x8 columns with the register
  *                  cap only (20 to 48 candidates);
- *   FV2 (scheme 2): the values 0 to 2 of dh_plan_set_variant_muscl;
+ *   FV2 (scheme 2): one candidate (the values of dh_plan_set_variant_muscl run
+ *                  the same tiles);
  *   FD (scheme 1): register cap x staging by asynchronous copies a variable at
- *                  a time or by TMA tensor copies (2 candidates, or 6 with TMA --
- *                  4 for GW59; TMA only when every level is a run of back-to-back
- *                  patches, see dh_plan_set_variant).
+ *                  a time or by TMA tensor copies (1 candidate for GW59, 2 for
+ *                  the others, 6 for the wave system when every level is a run
+ *                  of back-to-back patches, see dh_plan_set_variant).
  * `out` is overwritten.  If cache_path is NULL the environment variable
  * DH_TUNE_CACHE names the cache file (no cache when it is unset).  With a cache
  * file the choice is first looked up

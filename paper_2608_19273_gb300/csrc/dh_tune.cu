@@ -16,8 +16,8 @@
 //             x loads: plain (L2-prefetched) or, for 3D Euler, TMA tensor copies of every
 //               column plane and its ring strips into a double-buffered shared ring
 //   second-order FV stage: one form (the three values of its variant run the same tiles);
-//   FD stage: register cap (3 or 2 CTAs per SM) x staging (asynchronous copies or TMA);
-//             with TMA staging (systems of <= 5 variables) also caps for 3 and 4 CTAs per SM
+//   FD stage: register cap (3 or 2 CTAs per SM; one form for GW59); for the wave system also TMA
+//             staging, with caps for 1 to 4 CTAs per SM
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -80,8 +80,7 @@ struct Cand {
 static int tune_candidates(const dh_plan* plan, int scheme, Cand* cands) {
   int nc = 0;
   if (scheme == 2) {
-    // second-order FV: the three values run the same 8x8x4 tiles
-    for (int v = 0; v < 3; ++v) cands[nc++] = {v, plan->fv_zs, plan->fd_var};
+    cands[nc++] = {2, plan->fv_zs, plan->fd_var};  // (values 0 and 1 run the same 8x8x4 tiles)
     return nc;
   }
   if (scheme == 0) {
@@ -112,16 +111,11 @@ static int tune_candidates(const dh_plan* plan, int scheme, Cand* cands) {
           for (int vv = 2; vv < 4; ++vv) cands[nc++] = {32 | vv | (tile << 3), zz, plan->fd_var};
       }
   } else {
+    // only values that launch different kernels: GW59 has one, TMA staging is compiled for the wave system
     cands[nc++] = {plan->fv_var, plan->fv_zs, 0};
-    cands[nc++] = {plan->fv_var, plan->fv_zs, 2};
-    if (plan->tma_ok) {
-      cands[nc++] = {plan->fv_var, plan->fv_zs, 4};
-      cands[nc++] = {plan->fv_var, plan->fv_zs, 6};
-      if (plan->pde != DH_PDE_GW59) {
-        cands[nc++] = {plan->fv_var, plan->fv_zs, 12};
-        cands[nc++] = {plan->fv_var, plan->fv_zs, 20};
-      }
-    }
+    if (plan->pde != DH_PDE_GW59) cands[nc++] = {plan->fv_var, plan->fv_zs, 2};
+    if (plan->pde == DH_PDE_WAVE3D && plan->tma_ok)
+      for (int f : {4, 6, 12, 20}) cands[nc++] = {plan->fv_var, plan->fv_zs, f};
   }
   return nc;
 }

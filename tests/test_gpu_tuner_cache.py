@@ -66,3 +66,19 @@ def test_choice_saved_for_other_kernels_is_not_taken(tmp_path):
     cache.write_text(json.dumps(line) + "\n")
     choice = _tune(torch, mesh, synth.PDE_WAVE3D, 1, cache)
     assert not choice[3]
+
+
+@pytest.mark.parametrize("pde,scheme,halo,count", [(synth.PDE_EULER3D, 2, 2, 1), (synth.PDE_GW59, 1, 3, 1),
+                                                   (synth.PDE_ADV_NCP, 1, 3, 2), (synth.PDE_WAVE3D, 1, 3, 6)])
+def test_candidates_are_different_kernels(pde, scheme, halo, count):
+    """One candidate for each kernel that the values of a variant launch."""
+    torch = require_cuda()
+    mesh = _mesh(gap=False)
+    nq, nm = synth.PDE_NQ[pde], synth.PDE_NM[pde]
+    with dh.Plan(pde, 3, mesh.patches, halo, mesh.var_stride) as plan:
+        q = torch.ones((nq, mesh.var_stride), dtype=torch.float64, device="cuda")
+        q[nq - 1] = 2.5
+        mat = torch.full((nm, mesh.var_stride), 0.5, dtype=torch.float64, device="cuda") if nm else None
+        dt = torch.tensor([1e-3], dtype=torch.float64, device="cuda")
+        choice = dh.dh_autotune(plan, scheme, q, torch.empty_like(q), mat, dt, reps=1)
+        assert len([t for t in choice[4] if t > 0]) == count
