@@ -937,7 +937,7 @@ dh_status launch_fd_stage(dh_plan* plan, const double* qs, const double* q0, dou
   A.debug_no_issue = plan->debug_flags & 1;
   A.vs = plan->var_stride;
   A.P = plan->params;
-  if (plan->fd_var & 4) {
+  if ((plan->fd_var & 4) && plan->pde == DH_PDE_WAVE3D) {  // (the others run the ring, which reads no maps)
     if (!plan->tma_ok) { set_error("patch_update_fd_ko: the TMA variant needs contiguous levels (see dh_plan_create)"); return DH_EUNSUPPORTED; }
     dh_status st = encode_maps(plan, qs, A);
     if (st != DH_OK) return st;

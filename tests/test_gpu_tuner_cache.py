@@ -82,3 +82,23 @@ def test_candidates_are_different_kernels(pde, scheme, halo, count):
         dt = torch.tensor([1e-3], dtype=torch.float64, device="cuda")
         choice = dh.dh_autotune(plan, scheme, q, torch.empty_like(q), mat, dt, reps=1)
         assert len([t for t in choice[4] if t > 0]) == count
+
+
+@pytest.mark.parametrize("pde,same", [(synth.PDE_GW59, [(0, 2), (0, 4), (0, 6)]), (synth.PDE_ADV_NCP, [(0, 4), (2, 6), (0, 12), (0, 20)])])
+def test_values_that_share_a_kernel(pde, same):
+    """fd_var values that select TMA staging, for systems it is not compiled for: the ring's results bit for bit."""
+    torch = require_cuda()
+    mesh = _mesh(gap=False)
+    nq, nm = synth.PDE_NQ[pde], synth.PDE_NM[pde]
+    rng = np.random.default_rng(61)
+    q = torch.from_numpy(rng.uniform(0.5, 1.5, (nq, mesh.var_stride))).cuda()
+    mat = torch.from_numpy(rng.uniform(0.5, 1.5, (nm, mesh.var_stride))).cuda() if nm else None
+    dt = torch.tensor([1e-3], dtype=torch.float64, device="cuda")
+    outs = {}
+    with dh.Plan(pde, 3, mesh.patches, 3, mesh.var_stride) as plan:
+        for v in sorted({v for pair in same for v in pair}):
+            dh.dh_plan_set_variant(plan, 2, 0, v)
+            outs[v] = torch.zeros_like(q)
+            dh.patch_update_fd_ko(plan, q, None, outs[v], None, mat, dt, 0.0, 1.0, 1.0, 0.0, 0.1)
+    for a, b in same:
+        assert torch.equal(outs[a], outs[b])
