@@ -215,16 +215,15 @@ __global__ void k_check_sqrt(const double* x, double* y_sqrt, double* y_rsqrt, i
 static inline int pt_nbr(const dh_patch* patches, int k, int f) { return patches[k].nbr[f]; }
 
 // Work list of the generic FV stage (k_fv_any; see dh_fv_any.cuh).  An item's shape: ng groups
-// of bx x by x bz voxels; its limits: at most 256 voxels, 512 box cells with the face halo, 320
-// line cells and 256 faces of one direction.
+// of bx x by x bz voxels; its limits: at most 256 voxels, 512 box cells with the face halo and 256 faces
+// of one direction.
 static bool any_fits(int bx, int by, int bz, int ng, int dim) {
   const int ez = dim == 3 ? 2 : 0;
   if (ng < 1 || ng > 8 || bx < 1 || by < 1 || bz < 1 || (dim == 2 && bz != 1)) return false;
   if (ng * bx * by * bz > 256 || ng * (bx + 2) * (by + 2) * (bz + ez) > 512) return false;
   for (int d = 0; d < dim; ++d) {
-    const int lines = (bx + 2 * (d == 0)) * (by + 2 * (d == 1)) * (bz + 2 * (d == 2));
     const int faces = (bx + (d == 0)) * (by + (d == 1)) * (bz + (d == 2));
-    if (ng * lines > 320 || ng * faces > 256) return false;
+    if (ng * faces > 256) return false;
   }
   return true;
 }
