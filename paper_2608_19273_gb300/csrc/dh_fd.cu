@@ -387,7 +387,8 @@ __device__ bool tma_wait_all(const FdArgs& A, uint64_t* bar, uint32_t parity) {
 // waits for the other warps' arrival only when it needs i + 1, so that warps may be a variable apart, some
 // in integer stencils while others issue FP64 updates.  The box that new copies overwrite is that
 // of variable i - 2.  With __syncthreads for every variable (all warps in the same phase, one variable more
-// in flight) an RK4 step took 30.6 ms against 27.8 (GW59) and 4.36 against 3.98 (wave system).
+// in flight) an RK4 step took 30.6 ms against 27.8 (GW59) and 4.36 against 3.98 (wave system), with the
+// stencils of two guard bits.
 static_assert(FNSLOT == 4 * FNT, "four slots per thread");
 template <int NB>
 struct FdRing {
