@@ -490,7 +490,8 @@ dh_status dh_plan_create(dh_plan** out, int32_t pde, int32_t dim, const dh_patch
   // columns above 16 planes in chunks and a thin last wave in half-height chunks.  SSP-RK3
   // steps of 3D Euler against 16x16 columns without / with those chunks, us: 32 K voxels 362
   // against 871 / 459, 512 K 607 : 903 / 674, 27 patches of 24^3 489 : 1422 / 1415, 27 of 40^3 1927 : 3288 / 3290,
-  // 2.1 M voxels of 16^3 2373 : 2550 / 2329, 4.1 M 4362 : 4625 / 4439, the 10.5 M mix 10865 : 10951 / 11026.
+  // 2.1 M voxels of 16^3 2373 : 2550 / 2329, 4.1 M 4362 : 4625 / 4439, the 10.5 M mix 10865 : 10951 / 11026 (all before the pressures of a momentum sum became
+  // one term: 1.6% more).
   // SRHD, whose ring of halo voxels costs more (a wider W and three roots), is better off with 16x16
   // columns and those chunks once they fill one wave (two CTAs per SM): 110 K voxels 1194 : 1874 / 1319, 512 K
   // 1560 : 1904 / 1599, but 1.4 M 4413 : 4716 / 4196, 16.8 M 20.7 : 19.8 / 19.5 ms.
